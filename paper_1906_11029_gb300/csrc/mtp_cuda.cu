@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include "mtp_adjoint.cuh"
+#include "mtp_apex.cuh"
 #include "mtp_internal.h"
 #include "mtp_launch.cuh"
 
@@ -48,6 +49,8 @@ struct DeviceMesh {
     float* Lfr_lo = nullptr;
     float* Trf_lo = nullptr;
     float* Dtc = nullptr;         // tcgen05 A operand (variants 3, 4): D^T in core-matrix layout, hi then lo
+    void* ent = nullptr;          // apex tent kernel: patch entry records, change of basis
+    void* Rt = nullptr;
     double* partial = nullptr;    // energy reduction scratch: [n_rhs][kEnergyBlocks] partials, then [n_rhs] sums
 };
 
@@ -163,6 +166,103 @@ static void append_fragments(std::vector<float>& hi, std::vector<float>& lo, int
             }
 }
 
+// Records of the patch entries for the apex tent kernel (layout at kApexRec); one warp per vertex,
+// one lane per patch element, FP64 arithmetic, stored in the arithmetic precision.
+template <typename Real>
+__global__ void apex_record_kernel(int64_t nv, const int64_t* patch_ptr, const int32_t* patch_elem,
+                                   const int8_t* patch_info, const double* geo, Real* ent) {
+    const int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (v >= nv) return;
+    const int64_t pb = patch_ptr[v];
+    for (int64_t at = pb + (threadIdx.x & 31); at < patch_ptr[v + 1]; at += 32) {
+        const int8_t* info = patch_info + at * 12;
+        const double* g = geo + (int64_t)patch_elem[at] * kGeoStride;
+        const int j = info[0];
+        double gr[3][3], t[3][3];
+        for (int w = 0; w < 3; ++w)
+            for (int q = 0; q < 3; ++q) gr[w][q] = g[3 * (w < j ? w : w + 1) + q];
+        // edges from V: dual to the gradients of the other vertices' barycentric coordinates
+        double c[3][3];
+        for (int w = 0; w < 3; ++w) {
+            const double *x = gr[(w + 1) % 3], *y = gr[(w + 2) % 3];
+            c[w][0] = x[1] * y[2] - x[2] * y[1];
+            c[w][1] = x[2] * y[0] - x[0] * y[2];
+            c[w][2] = x[0] * y[1] - x[1] * y[0];
+        }
+        const double dg = gr[0][0] * c[0][0] + gr[0][1] * c[0][1] + gr[0][2] * c[0][2];
+        const double s = g[28], l = exp2(rint(log2(1.0 / (s * s)) / 3.0));
+        for (int w = 0; w < 3; ++w)
+            for (int q = 0; q < 3; ++q) {
+                t[w][q] = c[w][q] / dg / l;
+                gr[w][q] *= l;
+            }
+        const double det = 1.0 / (dg * l * l * l), ts = l * s, sgn = det > 0 ? 1.0 : -1.0;
+        Real* r = ent + at * kApexRec;
+        auto dot = [](const double* x, const double* y) { return x[0] * y[0] + x[1] * y[1] + x[2] * y[2]; };
+        int n = 0;
+        double G[3][3];
+        for (int w = 0; w < 3; ++w)
+            for (int x = w; x < 3; ++x, ++n) {
+                G[w][x] = G[x][w] = dot(t[w], t[x]);
+                r[n] = (Real)G[w][x];
+                r[6 + n] = (Real)dot(gr[w], gr[x]);
+            }
+        r[12] = (Real)(1.0 / l);
+        r[13] = (Real)g[29];
+        r[14] = (Real)g[30];
+        r[15] = (Real)det;
+        r[16] = (Real)(1.0 / (l * det));
+        r[17] = (Real)(ts * l * det);
+        r[18] = (Real)(1.0 / (l * det * ts));
+        r[19] = (Real)(1.0 / (g[29] * g[30]));
+        for (int fi = 0; fi < 3; ++fi) {
+            const int X = fi == 0 ? 1 : 0, Y = fi == 2 ? 1 : 2;
+            const int s2 = info[4 + (fi < j ? fi : fi + 1)];
+            const double zm = g[31], zp = s2 >= 0 ? geo[(int64_t)patch_elem[pb + s2] * kGeoStride + 31] : zm;
+            const double area = sqrt(G[X][X] * G[Y][Y] - G[X][Y] * G[X][Y]), q = sgn / (area * (zm + zp));
+            Real* o = r + kApexFacet + 6 * fi;
+            o[0] = (Real)(zm / (zm + zp));
+            o[1] = (Real)(zp / (zm + zp));
+            o[2] = (Real)(q * G[Y][Y]);
+            o[3] = (Real)(-q * G[X][Y]);
+            o[4] = (Real)(q * G[X][X]);
+            o[5] = (Real)(zm * zp);
+        }
+        for (int w = 0; w < 3; ++w)
+            for (int q = 0; q < 3; ++q) {
+                r[kApexDual + 3 * w + q] = (Real)gr[w][q];
+                r[kApexEdge + 3 * w + q] = (Real)t[w][q];
+            }
+    }
+}
+
+template <typename Real>
+static int apex_upload_real(const Mesh& m, DeviceMesh& d) {
+    std::vector<Real> rt;
+    const int nb = m.nb;
+    for (int j = 0; j < 4; ++j)
+        for (int k = 0, b0 = 0; k <= m.p; b0 += apex_rot_block(k), ++k) {
+            const int n = apex_rot_block(k);
+            for (int a = 0; a < n; ++a)
+                for (int b = 0; b < pad4(n); ++b)
+                    rt.push_back(b < n ? (Real)m.ref.Rot[((size_t)j * nb + b0 + a) * nb + b0 + b] : Real(0));
+        }
+    MTP_TRY(upload((Real**)&d.Rt, rt.data(), rt.size()));
+    CUDA_TRY(cudaMalloc(&d.ent, m.patch_elem.size() * kApexRec * sizeof(Real) + 16));
+    const int64_t blocks = (m.nv * 32 + 127) / 128;
+    apex_record_kernel<Real><<<(unsigned)blocks, 128>>>(m.nv, d.patch_ptr, d.patch_elem, d.patch_info, d.geo, (Real*)d.ent);
+    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(cudaDeviceSynchronize());   // later launches may use any stream
+    return MTP_OK;
+}
+
+// the apex tent kernel runs the plain SAT modes in 3D up to kApexMaxDegree
+static int apex_upload(const Mesh& m, DeviceMesh& d) {
+    if (m.dim != 3 || m.p > kApexMaxDegree) return MTP_OK;
+    if (m.precision == MTP_FP64) return apex_upload_real<double>(m, d);
+    return m.precision == MTP_FP32 ? apex_upload_real<float>(m, d) : MTP_OK;
+}
+
 int device_mesh_upload(Mesh& m) {
     int dev;
     CUDA_TRY(cudaGetDevice(&dev));
@@ -245,6 +345,7 @@ int device_mesh_upload(Mesh& m) {
         MTP_TRY(upload(&d.Lfr_lo, ll.data(), ll.size()));
         MTP_TRY(upload(&d.Trf_lo, tl.data(), tl.size()));
     }
+    MTP_TRY(apex_upload(m, d));
     MTP_TRY(upload(&d.V, m.ref.V.data(), m.ref.V.size()));
     MTP_TRY(upload(&d.Vinv, m.ref.Vinv.data(), m.ref.Vinv.size()));
     CUDA_TRY(cudaMalloc((void**)&d.partial, sizeof(double) * (kEnergyBlocks + 1) * m.n_rhs));
@@ -256,7 +357,7 @@ void device_mesh_free(Mesh& m) {
     DeviceMesh& d = *m.dev;
     void* ptrs[] = {d.geo, d.elems, d.patch_ptr, d.patch_elem, d.patch_info, d.S, d.Tr, d.L, d.Mc, d.Dc, d.Trc, d.Lc, d.Mc1, d.Dc1, d.Trc1, d.Lc1,
                     d.V, d.Vinv, d.partial,
-                    d.Sf, d.Lfr, d.Trf, d.Sf_lo, d.Lfr_lo, d.Trf_lo, d.Dtc};
+                    d.Sf, d.Lfr, d.Trf, d.Sf_lo, d.Lfr_lo, d.Trf_lo, d.Dtc, d.ent, d.Rt};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete m.dev;
@@ -508,6 +609,8 @@ static void fill_args(Tents& t, void* state, KArgs& a) {
     a.Lfr_lo = (const float4*)dm.Lfr_lo;
     a.Trf_lo = (const float4*)dm.Trf_lo;
     a.Dtc = dm.Dtc;
+    a.ent = dm.ent;
+    a.Rt = dm.Rt;
     a.state = state;
     a.rhs_stride = m.ne * m.nf * m.nb;
     a.err = dt.err;
@@ -580,7 +683,12 @@ int device_evolve(Tents& t, void* state, int64_t lb, int64_t le, bool use_graph,
         CUDA_TRY(ke.persistent_prepare(m.max_patch, &bpsm));
         CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
         const int64_t t0 = t.layer_ptr[lb], nt = t.layer_ptr[le] - t0;
-        const int cps = launch == 1 ? 1 : std::max(1, bpsm);
+        // as many CTAs per SM as fit, but no more than the layers fill: CTAs beyond the tents of a
+        // layer only wait, and leave the running ones unevenly spread over the SMs (cavity 16^3,
+        // p = 3, 133 tents per layer: 73 us per layer with 3 CTAs per SM, 61 us with one)
+        const double width = (double)nt / (double)(le - lb);
+        const int fill = (int)std::min(64.0, std::ceil(width / nsm));
+        const int cps = launch == 1 ? 1 : std::max(1, std::min(bpsm, fill));
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t)cps * nsm));
         if (lb == 0) {
             CUDA_TRY(cudaMemsetAsync(d.cnt, 0, sizeof(int) * m.nv, st));
@@ -845,7 +953,10 @@ int device_batch_evolve(Batch& b, void* const* states, void* stream) {
             return set_error(MTP_EUNSUPPORTED, "batches run SAT meshes; MTP_FLAG_SUBSTITUTED_RK4 is per mesh");
     if (m0.precision == MTP_TF32 || m0.precision == MTP_TF32X3 || m0.precision == MTP_FP32_SPLIT)
         return set_error(MTP_EUNSUPPORTED, "batches run FP64 or FP32 SIMT meshes; tensor-core and split modes are per mesh");
-    const BatchEntry& be = table[m0.precision == MTP_FP64 ? 0 : 1][m0.dim - 2];
+    int pmax = 0;
+    for (Tents* t : b.inst) pmax = std::max(pmax, t->mesh->p);
+    BatchEntry be = table[m0.precision == MTP_FP64 ? 0 : 1][m0.dim - 2];
+    if (m0.dim == 3 && pmax <= kApexMaxDegree) be = m0.precision == MTP_FP64 ? apex_batch_f64(pmax) : apex_batch_f32(pmax);
     if (!b.dev) {
         b.dev = new DeviceBatch();
         DeviceBatch& d = *b.dev;

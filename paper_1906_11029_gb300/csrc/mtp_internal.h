@@ -12,6 +12,7 @@ namespace mtp {
 constexpr int kMaxDegree = 5;
 constexpr int kMaxPatch3D = 32;   // Kuhn/Freudenthal meshes have 24 tets per interior vertex
 constexpr int kMaxPatch2D = 16;
+constexpr int kApexMaxDegree = 4;   // degrees of the apex tent kernel (3D)
 
 inline int n_basis(int dim, int p) {
     return dim == 2 ? (p + 1) * (p + 2) / 2 : (p + 1) * (p + 2) * (p + 3) / 6;
@@ -35,6 +36,10 @@ struct RefTables {
     std::vector<double> Tr;
     // L[j][f][a][c] = int_{F^} lambda_j(x_f(s)) psi_a(x_f(s)) chi_c(s) ds
     std::vector<double> L;
+    // 3D, p <= kApexMaxDegree: Rot[j][a][b] = int psi'_a psi_b with psi' the basis on the element
+    // whose collapsed apex is local vertex j (coordinates: the other vertices in ascending order
+    // take the places C, D, B of the apex tent kernel); orthogonal, block-diagonal in the degree
+    std::vector<double> Rot;
     // V[k][a] = psi_a(lattice point k), Vinv its inverse
     std::vector<double> V, Vinv;
     double max_orth_err = 0;   // max |int psi_a psi_b - delta_ab| (diagnostic)

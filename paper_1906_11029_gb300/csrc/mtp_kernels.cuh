@@ -68,6 +68,10 @@ struct KArgs {
     // tcgen05 volume operator (shapes v = 3, 4): A operand D^T[a][(l, c)] (rows a padded to 64)
     // in the K-major core-matrix layout, TF32 hi part then lo part, each 64 x TK floats
     const float* Dtc;
+    // apex tent kernel (3D, p <= 4, see mtp_apex.cuh): geometry record of every patch entry and
+    // the change of basis per local index of V
+    const void* ent;
+    const void* Rt;
     void* state;                // [rhs][ne][nf][nb]
     int64_t rhs_stride;         // ne * nf * nb
     int* err;                   // error word (0 = ok, 1 = causality, 2 = non-finite)
@@ -1377,20 +1381,13 @@ __device__ __forceinline__ long long globaltimer() {
     return t;
 }
 
-// One DAG-walk step for ticket `tent` of an instance: bounded wait on the closed neighbourhood,
-// all right-hand sides, publish.  Returns false when the CTA must stop (error / timeout).
-template <typename Real, int DIM, int P, int MODE = 0>
-__device__ bool tent_dag_step(unsigned char* smem, const KArgs& a, const PArgs& pa, int64_t tent, int* s_abort) {
-    using Sh = Shape<DIM, P>;
-    using StateT = StateOf<Real, MODE>;
-    constexpr int NF = Sh::NF, NB = Sh::NB, NT = Sh::NT, NBP = Sh::NBP, ESZ = NF * NBP;
-    const SmemLayout<Real, DIM, P> lay(a.max_patch, MODE);
-    TentCtx<Real, DIM, P> c;
-    c.carve(smem, lay);
+// All threads: bounded wait until the closed neighbourhood of the tent's vertex has completed its
+// tents of earlier layers.  Returns false when the CTA must stop (error / timeout).
+__device__ __forceinline__ bool dag_wait(const KArgs& a, const PArgs& pa, int64_t tent, int* s_abort) {
     const int V = a.tent_v[tent];
     const int L = pa.tent_layer[tent];
     const int64_t a0 = pa.adj_ptr[V], deg = pa.adj_ptr[V + 1] - a0;
-    for (int u = threadIdx.x; u <= deg; u += NT) {
+    for (int u = threadIdx.x; u <= deg; u += blockDim.x) {
         const int U = u == 0 ? V : pa.adj[a0 + u - 1];
         int64_t lo = pa.vt_ptr[U], hi = pa.vt_ptr[U + 1];
         const int64_t base = lo;
@@ -1412,7 +1409,31 @@ __device__ bool tent_dag_step(unsigned char* smem, const KArgs& a, const PArgs& 
         }
     }
     __syncthreads();
-    if (*s_abort) return false;
+    return *s_abort == 0;
+}
+
+// One thread, after a barrier behind every thread's __threadfence(): advance the front at V and
+// publish the tent's completion.
+__device__ __forceinline__ void dag_publish(const KArgs& a, const PArgs& pa, int64_t tent) {
+    if (threadIdx.x == 0 && !(pa.withhold_first && tent == pa.ticket0)) {
+        const int V = a.tent_v[tent];
+        a.tau[V] = a.tent_tt[tent];
+        __threadfence();
+        atomicAdd(pa.cnt + V, 1);
+    }
+}
+
+// One DAG-walk step for ticket `tent` of an instance: bounded wait on the closed neighbourhood,
+// all right-hand sides, publish.  Returns false when the CTA must stop (error / timeout).
+template <typename Real, int DIM, int P, int MODE = 0>
+__device__ bool tent_dag_step(unsigned char* smem, const KArgs& a, const PArgs& pa, int64_t tent, int* s_abort) {
+    using Sh = Shape<DIM, P>;
+    using StateT = StateOf<Real, MODE>;
+    constexpr int NF = Sh::NF, NB = Sh::NB, NT = Sh::NT, NBP = Sh::NBP, ESZ = NF * NBP;
+    const SmemLayout<Real, DIM, P> lay(a.max_patch, MODE);
+    TentCtx<Real, DIM, P> c;
+    c.carve(smem, lay);
+    if (!dag_wait(a, pa, tent, s_abort)) return false;
     for (int r = 0; r < pa.n_rhs; ++r) {
         StateT* state = (StateT*)a.state + (int64_t)r * a.rhs_stride;
         tent_setup<Real, DIM, P, true>(c, a, tent, state);
@@ -1429,11 +1450,7 @@ __device__ bool tent_dag_step(unsigned char* smem, const KArgs& a, const PArgs& 
         __threadfence();                       // publish this thread's state writes (gpu scope)
         __syncthreads();
     }
-    if (threadIdx.x == 0 && !(pa.withhold_first && tent == pa.ticket0)) {
-        a.tau[V] = a.tent_tt[tent];
-        __threadfence();
-        atomicAdd(pa.cnt + V, 1);
-    }
+    dag_publish(a, pa, tent);
     __syncthreads();
     return true;
 }

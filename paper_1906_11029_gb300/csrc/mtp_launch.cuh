@@ -81,6 +81,10 @@ void kernel_table_f32_v2(KernelEntry entries[2][5]);
 // FP32 3D, volume term on tcgen05 (variants 3 and 4, p = 2..4): entries[variant - 3][p - 1]
 void kernel_table_f32_tc5(KernelEntry entries[2][5]);
 
+// apex tent kernel, 3D, p <= kApexMaxDegree (mtp_apex.cuh)
+KernelEntry apex_entry_f32(int p);
+KernelEntry apex_entry_f64(int p);
+
 struct AdjArgs;
 using AdjLaunchFn = cudaError_t (*)(const AdjArgs&, int64_t t0, int n_tents, int n_rhs, cudaStream_t st);
 using TapeStrideFn = int64_t (*)(int max_patch, int m, int q);
@@ -102,6 +106,9 @@ struct BatchEntry {
 };
 // entries[precision][dim - 2]
 void batch_table(BatchEntry entries[2][2]);
+// 3D batches whose largest degree is at most kApexMaxDegree
+BatchEntry apex_batch_f32(int pmax);
+BatchEntry apex_batch_f64(int pmax);
 
 #define MTP_KERNEL_ENTRY(REAL, D, P, MODE)                                                      \
     KernelEntry{launch_tent_kernel<REAL, D, P, MODE>, prepare_tent_kernel<REAL, D, P, MODE>,     \

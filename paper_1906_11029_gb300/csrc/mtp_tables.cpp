@@ -355,6 +355,23 @@ RefTables build_ref_tables(int d, int p) {
                     if (!(std::fabs((double)acc - t.S[(((size_t)j * d + l) * nb + a) * nb + b]) <= 1e-12 * smax))
                         throw std::runtime_error("reference tables: factored volume tables do not reproduce S");
                 }
+    if (d == 3 && p <= kApexMaxDegree) {
+        t.Rot.assign((size_t)(d + 1) * nb * nb, 0.0);
+        for (int j = 0; j <= d; ++j) {
+            std::vector<Poly> at;   // coordinates x, y, z of the apex frame: lambda_D, lambda_B, lambda_A
+            for (int i = 0, n = 0; i <= d; ++i)
+                if (i != j && n++ > 0) at.push_back(lam[i]);
+            at.push_back(lam[j]);
+            for (int a = 0; a < nb; ++a) {
+                const Poly r = compose(psi[a], at[0], at[1], at[2]);
+                for (int b = 0; b < nb; ++b) {
+                    double& v = t.Rot[((size_t)j * nb + a) * nb + b];
+                    v = (double)integrate(mul(r, psi[b]), d);
+                    if (dpsi_deg[a] != dpsi_deg[b]) zero(v, 1.0);
+                }
+            }
+        }
+    }
     // lattice Vandermonde (point order: i_d outermost, i_1 innermost)
     std::vector<ld> V((size_t)nb * nb);
     int k = 0;
