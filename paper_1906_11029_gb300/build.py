@@ -24,8 +24,8 @@ CUDA_HOME = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 NVCC = os.path.join(CUDA_HOME, "bin", "nvcc")
 GENCODE = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CXX_SOURCES = ["mtp_host.cpp", "mtp_tables.cpp"]
-CU_SOURCES = ["mtp_cuda.cu", "mtp_k64.cu", "mtp_k32.cu", "mtp_ka32.cu", "mtp_ka64.cu", "mtp_kab32.cu", "mtp_kab64.cu", "mtp_ks.cu", "mtp_krk.cu", "mtp_kv.cu", "mtp_kv2.cu", "mtp_ktc5.cu", "mtp_ktc.cu", "mtp_kb.cu", "mtp_adj.cu", "mtp_probe.cu", "mtp_noalloc.cu", "mtp_pitch.cu"]
-HEADERS = ["mtp_internal.h", "mtp_kernels.cuh", "mtp_apex.cuh", "mtp_apex_launch.cuh", "mtp_adjoint.cuh", "mtp_launch.cuh", "../../include/mtp.h"]
+CU_SOURCES = ["mtp_cuda.cu", "mtp_lattice.cu", "mtp_k64.cu", "mtp_k32.cu", "mtp_ka32.cu", "mtp_ka64.cu", "mtp_kab32.cu", "mtp_kab64.cu", "mtp_ks.cu", "mtp_krk.cu", "mtp_kv.cu", "mtp_kv2.cu", "mtp_ktc5.cu", "mtp_ktc.cu", "mtp_kb.cu", "mtp_adj.cu", "mtp_probe.cu", "mtp_noalloc.cu", "mtp_pitch.cu"]
+HEADERS = ["mtp_internal.h", "mtp_device.h", "mtp_kernels.cuh", "mtp_apex.cuh", "mtp_apex_launch.cuh", "mtp_adjoint.cuh", "mtp_launch.cuh", "../../include/mtp.h"]
 
 
 def _newer(src_list, target):
@@ -54,12 +54,12 @@ def build(verbose: bool = False, force: bool = False, ptxas_info: bool = False) 
     jobs, objs = [], []
     cxx = shutil.which("g++") or "g++"
     # straight-line contractions of the apex tent kernel, written by a small host program
-    gen, ops = (os.path.join(BUILD, s) for s in ("apexgen", "mtp_apex_ops.h"))
+    gen, ops, lat = (os.path.join(BUILD, s) for s in ("apexgen", "mtp_apex_ops.h", "mtp_lattice_ops.h"))
     gen_src = [os.path.join(CSRC, s) for s in ("mtp_apexgen.cpp", "mtp_tables.cpp", "mtp_internal.h")]
-    if force or _newer(gen_src, ops):
+    if force or _newer(gen_src, ops) or _newer(gen_src, lat):
         _run([cxx, "-O2", "-std=c++17", "-Wno-unused-function", *inc, gen_src[0], "-o", gen])
-        _run([gen, ops])
-    headers.append(ops)
+        _run([gen, ops, lat])
+    headers += [ops, lat]
     for s in CXX_SOURCES:
         src = os.path.join(CSRC, s)
         obj = os.path.join(BUILD, s + ".o")

@@ -8,6 +8,12 @@
 // at p = 4 multiplication by lambda_V has 50 non-zeros of 700, the derivatives along three suitable
 // directions 108, 112 and 144 of 700, the trace onto a facet through V 105 of 525, or 105 + 105 in
 // two factors.  Only the non-zeros are written out, so a thread needs no table loads and no loop.
+//
+// A second header, mtp_lattice_ops.h, holds the lattice Vandermonde matrix V and its inverse of
+// every dimension and degree in the same form.  Exchanging the element's first two vertices maps
+// the lattice onto itself and multiplies a basis function by +-1, so values at mirrored points are
+// the sum and the difference of an even and an odd part: 653 multiply-adds instead of 1225 at
+// p = 4 in 3D.
 #include <cstdio>
 #include <string>
 
@@ -173,14 +179,89 @@ void emit_degree(FILE* f, int p) {
     std::fprintf(f, "};\n\n");
 }
 
+void emit_lattice(FILE* f, int d, int p) {
+    const RefTables t = build_ref_tables(d, p);
+    const int nb = t.nb;
+    std::vector<int> pt;                       // integer coordinates, lattice order
+    for (int c = 0; c <= (d == 3 ? p : 0); ++c)
+        for (int b = 0; b + c <= p; ++b)
+            for (int a = 0; a + b + c <= p; ++a) pt.insert(pt.end(), {a, b, c});
+    std::vector<int> mirror(nb), sg(nb, 0);
+    for (int k = 0; k < nb; ++k)
+        for (int l = 0; l < nb; ++l)
+            if (pt[3 * l] == p - pt[3 * k] - pt[3 * k + 1] - pt[3 * k + 2] && pt[3 * l + 1] == pt[3 * k + 1] &&
+                pt[3 * l + 2] == pt[3 * k + 2])
+                mirror[k] = l;
+    for (int a = 0; a < nb; ++a)
+        for (int k = 0; k < nb; ++k) {
+            const double x = t.V[(size_t)k * nb + a], y = t.V[(size_t)mirror[k] * nb + a];
+            if (std::fabs(x) < 1e-9) continue;
+            const int s = x * y > 0 ? 1 : -1;
+            if (std::fabs(x - s * y) > 1e-10 || (sg[a] && sg[a] != s)) throw std::runtime_error("lattice mirror symmetry violated");
+            sg[a] = s;
+        }
+    auto lit = [](double v) {
+        char b[40];
+        std::snprintf(b, sizeof b, "%.17g", v);
+        return std::string(b);
+    };
+    std::fprintf(f, "template <>\nstruct LatticeOps<%d, %d> {\n", d, p);
+    std::fprintf(f, "    template <typename Put>\n    static __device__ __forceinline__ void to(const double* x, Put put) {\n        double e, o;\n");
+    for (int k = 0; k < nb; ++k) {
+        if (mirror[k] < k) continue;
+        std::string e, o;
+        for (int a = 0; a < nb; ++a) {
+            const double v = t.V[(size_t)k * nb + a];
+            if (std::fabs(v) < 1e-13) continue;
+            std::string& s = sg[a] > 0 ? e : o;
+            s = s.empty() ? lit(v) + " * x[" + std::to_string(a) + "]" : "__fma_rn(" + lit(v) + ", x[" + std::to_string(a) + "], " + s + ")";
+        }
+        if (mirror[k] == k) {
+            std::fprintf(f, "        put(%d, %s);\n", k, e.c_str());
+        } else {
+            std::fprintf(f, "        e = %s;\n        o = %s;\n        put(%d, e + o);\n        put(%d, e - o);\n", e.c_str(), o.c_str(), k, mirror[k]);
+        }
+    }
+    std::fprintf(f, "    }\n    template <typename Put>\n    static __device__ __forceinline__ void from(double* v, Put put) {\n        double t;\n");
+    for (int k = 0; k < nb; ++k)               // sums in place of the first, differences of the second
+        if (mirror[k] > k)
+            std::fprintf(f, "        t = v[%d] - v[%d];\n        v[%d] += v[%d];\n        v[%d] = t;\n", k, mirror[k], k, mirror[k], mirror[k]);
+    for (int a = 0; a < nb; ++a) {
+        std::string s;
+        for (int k = 0; k < nb; ++k) {
+            if (mirror[k] < k || (sg[a] < 0 && mirror[k] == k)) continue;
+            const double w = t.Vinv[(size_t)a * nb + k], w2 = t.Vinv[(size_t)a * nb + mirror[k]];
+            const double c = mirror[k] == k ? w : 0.5 * (w + sg[a] * w2);
+            const std::string x = "v[" + std::to_string(sg[a] > 0 ? k : mirror[k]) + "]";
+            s = s.empty() ? lit(c) + " * " + x : "__fma_rn(" + lit(c) + ", " + x + ", " + s + ")";
+        }
+        std::fprintf(f, "        put(%d, %s);\n", a, s.c_str());
+    }
+    // every entry, in the order of the points
+    std::fprintf(f, "    }\n    template <typename Put>\n    static __device__ __forceinline__ void from_dense(const double* v, Put put) {\n");
+    for (int a = 0; a < nb; ++a) {
+        std::string s = lit(t.Vinv[(size_t)a * nb]) + " * v[0]";
+        for (int k = 1; k < nb; ++k) s = "__fma_rn(" + lit(t.Vinv[(size_t)a * nb + k]) + ", v[" + std::to_string(k) + "], " + s + ")";
+        std::fprintf(f, "        put(%d, %s);\n", a, s.c_str());
+    }
+    std::fprintf(f, "    }\n};\n\n");
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
-    if (argc != 2) return 2;
+    if (argc != 3) return 2;
     FILE* f = std::fopen(argv[1], "w");
     if (!f) return 1;
     std::fprintf(f, "// generated by mtp_apexgen.cpp\n#pragma once\n\nnamespace mtp {\n\ntemplate <int P>\nstruct ApexOps;\n\n");
     for (int p = 1; p <= 4; ++p) emit_degree(f, p);
+    std::fprintf(f, "}  // namespace mtp\n");
+    if (std::fclose(f)) return 1;
+    f = std::fopen(argv[2], "w");
+    if (!f) return 1;
+    std::fprintf(f, "// generated by mtp_apexgen.cpp\n#pragma once\n\nnamespace mtp {\n\ntemplate <int DIM, int P>\nstruct LatticeOps;\n\n");
+    for (int d = 2; d <= 3; ++d)
+        for (int p = 1; p <= kMaxDegree; ++p) emit_lattice(f, d, p);
     std::fprintf(f, "}  // namespace mtp\n");
     return std::fclose(f) ? 1 : 0;
 }

@@ -1,5 +1,4 @@
-// Device-side management of the MTP library: uploads, lattice exchange, energy,
-// and the layer-by-layer evolution driver (layers replayed from a CUDA graph).
+// Device-side management of the MTP library: uploads and the evolution drivers.
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -9,18 +8,11 @@
 
 #include "mtp_adjoint.cuh"
 #include "mtp_apex.cuh"
+#include "mtp_device.h"
 #include "mtp_internal.h"
 #include "mtp_launch.cuh"
 
 namespace mtp {
-
-#define CUDA_TRY(call)                                                                       \
-    do {                                                                                     \
-        cudaError_t _e = (call);                                                             \
-        if (_e != cudaSuccess)                                                               \
-            return set_error(_e == cudaErrorMemoryAllocation ? MTP_ENOMEM : MTP_ECUDA,       \
-                             std::string(#call) + ": " + cudaGetErrorString(_e));            \
-    } while (0)
 
 struct DeviceMesh {
     int device = -1;
@@ -40,8 +32,6 @@ struct DeviceMesh {
     void* Dc1 = nullptr;
     void* Trc1 = nullptr;
     void* Lc1 = nullptr;
-    double* V = nullptr;
-    double* Vinv = nullptr;
     float* Sf = nullptr;          // tensor-core fragment tables (TF32 modes)
     float* Lfr = nullptr;
     float* Trf = nullptr;
@@ -80,12 +70,6 @@ struct DeviceTents {
     int64_t* tent_off = nullptr;   // [n_tents + 1]: patch entries of the tents before each tent
 };
 
-constexpr int kEnergyBlocks = 304;
-constexpr int kEnergyThreads = 256;
-
-// the state between tents is FP64 for MTP_FP64 and MTP_FP32_SPLIT, FP32 otherwise; the reference
-// tables and the tent kernels' arithmetic are FP64 only for MTP_FP64
-static bool state_f64(const Mesh& m) { return m.precision == MTP_FP64 || m.precision == MTP_FP32_SPLIT; }
 static size_t real_size(const Mesh& m) { return state_f64(m) ? sizeof(double) : sizeof(float); }
 
 template <typename T>
@@ -130,12 +114,6 @@ static int upload_real(const Mesh& m, void** dst, const std::vector<double>& src
     std::vector<float> f(src.begin(), src.end());
     return upload((float**)dst, f.data(), f.size());
 }
-
-#define MTP_TRY(call)                  \
-    do {                               \
-        int _rc = (call);              \
-        if (_rc != MTP_OK) return _rc; \
-    } while (0)
 
 // A-operand tables in m16n8k8 fragment order: fragment (mt, kt) of a row-major M x K matrix
 // A (zero outside rows < rows, cols < cols) is 32 lanes x 4 values: lane (g = lane/4,
@@ -346,9 +324,7 @@ int device_mesh_upload(Mesh& m) {
         MTP_TRY(upload(&d.Trf_lo, tl.data(), tl.size()));
     }
     MTP_TRY(apex_upload(m, d));
-    MTP_TRY(upload(&d.V, m.ref.V.data(), m.ref.V.size()));
-    MTP_TRY(upload(&d.Vinv, m.ref.Vinv.data(), m.ref.Vinv.size()));
-    CUDA_TRY(cudaMalloc((void**)&d.partial, sizeof(double) * (kEnergyBlocks + 1) * m.n_rhs));
+    CUDA_TRY(cudaMalloc((void**)&d.partial, sizeof(double) * energy_scratch_doubles(m)));
     return MTP_OK;
 }
 
@@ -356,7 +332,7 @@ void device_mesh_free(Mesh& m) {
     if (!m.dev) return;
     DeviceMesh& d = *m.dev;
     void* ptrs[] = {d.geo, d.elems, d.patch_ptr, d.patch_elem, d.patch_info, d.S, d.Tr, d.L, d.Mc, d.Dc, d.Trc, d.Lc, d.Mc1, d.Dc1, d.Trc1, d.Lc1,
-                    d.V, d.Vinv, d.partial,
+                    d.partial,
                     d.Sf, d.Lfr, d.Trf, d.Sf_lo, d.Lfr_lo, d.Trf_lo, d.Dtc, d.ent, d.Rt};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -438,139 +414,8 @@ static const KernelEntry& kernel_entry(const Mesh& m, int variant = 0) {
 }
 
 
-// ---------------------------------------------------------------------------------
-// lattice exchange: y(x_k) = (1/sqrt|det J|) sum_a V[k][a] Y_a and its inverse
-// ---------------------------------------------------------------------------------
-template <typename Real>
-__global__ void from_lattice_kernel(const double* vals, Real* state, const double* geo, const double* Vinv,
-                                    int64_t ne, int nf, int nb, int nrhs) {
-    const int64_t n = (int64_t)nrhs * ne * nb;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t re = i / nb;
-        const int a = (int)(i - re * nb);
-        const int64_t e = re % ne;
-        const double sq = 1.0 / geo[e * kGeoStride + 28];
-        const double* v = vals + re * nb * nf;
-        for (int f = 0; f < nf; ++f) {
-            double acc = 0;
-            for (int k = 0; k < nb; ++k) acc += Vinv[a * nb + k] * v[k * nf + f];
-            state[(re * nf + f) * nb + a] = (Real)(sq * acc);
-        }
-    }
-}
-
-template <typename Real>
-__global__ void to_lattice_kernel(const Real* state, double* vals, const double* geo, const double* V,
-                                  int64_t ne, int nf, int nb, int nrhs) {
-    const int64_t n = (int64_t)nrhs * ne * nb;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t re = i / nb;
-        const int k = (int)(i - re * nb);
-        const int64_t e = re % ne;
-        const double is = geo[e * kGeoStride + 28];
-        for (int f = 0; f < nf; ++f) {
-            double acc = 0;
-            for (int a = 0; a < nb; ++a) acc += V[k * nb + a] * (double)state[(re * nf + f) * nb + a];
-            vals[(re * nb + k) * nf + f] = is * acc;
-        }
-    }
-}
-
-static int grid_for(int64_t n, int threads) {
-    int64_t g = (n + threads - 1) / threads;
-    if (g > 152 * 64) g = 152 * 64;
-    return (int)(g < 1 ? 1 : g);
-}
-
-int device_from_lattice(Mesh& m, const double* vals, void* state, void* stream) {
-    MTP_TRY(device_mesh_upload(m));
-    cudaStream_t st = (cudaStream_t)stream;
-    const int64_t n = (int64_t)m.n_rhs * m.ne * m.nb;
-    if (state_f64(m))
-        from_lattice_kernel<double><<<grid_for(n, 256), 256, 0, st>>>(vals, (double*)state, m.dev->geo, m.dev->Vinv,
-                                                                       m.ne, m.nf, m.nb, m.n_rhs);
-    else
-        from_lattice_kernel<float><<<grid_for(n, 256), 256, 0, st>>>(vals, (float*)state, m.dev->geo, m.dev->Vinv,
-                                                                      m.ne, m.nf, m.nb, m.n_rhs);
-    CUDA_TRY(cudaGetLastError());
-    return MTP_OK;
-}
-
-int device_to_lattice(Mesh& m, const void* state, double* vals, void* stream) {
-    MTP_TRY(device_mesh_upload(m));
-    cudaStream_t st = (cudaStream_t)stream;
-    const int64_t n = (int64_t)m.n_rhs * m.ne * m.nb;
-    if (state_f64(m))
-        to_lattice_kernel<double><<<grid_for(n, 256), 256, 0, st>>>((const double*)state, vals, m.dev->geo, m.dev->V,
-                                                                     m.ne, m.nf, m.nb, m.n_rhs);
-    else
-        to_lattice_kernel<float><<<grid_for(n, 256), 256, 0, st>>>((const float*)state, vals, m.dev->geo, m.dev->V,
-                                                                    m.ne, m.nf, m.nb, m.n_rhs);
-    CUDA_TRY(cudaGetLastError());
-    return MTP_OK;
-}
-
-// ---------------------------------------------------------------------------------
-// energy on a flat front: 1/2 sum (|Y_E|^2/eps + |Y_H|^2/mu); two-pass deterministic
-// reduction through the per-block partials buffer
-// ---------------------------------------------------------------------------------
-template <typename Real>
-__global__ void energy_partial_kernel(const Real* state, const double* geo, int64_t ne, int nf, int nb,
-                                      double* partial) {
-    __shared__ double red[kEnergyThreads];
-    const int rhs = blockIdx.y;
-    const Real* s = state + (int64_t)rhs * ne * nf * nb;
-    const int64_t n = ne * nf * nb;
-    double acc = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t e = i / (nf * nb);
-        const int f = (int)((i / nb) % nf);
-        const double y = (double)s[i];
-        const double* g = geo + e * kGeoStride;
-        const bool isE = nf == 6 ? f < 3 : f < 2;   // E fields first, then H (2D: Ex, Ey | Hz)
-        acc += y * y / (isE ? g[29] : g[30]);
-    }
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partial[rhs * gridDim.x + blockIdx.x] = red[0];
-}
-
-__global__ void energy_final_kernel(const double* partial, int nblocks, double* out) {
-    __shared__ double red[kEnergyThreads];
-    const int rhs = blockIdx.x;
-    double acc = 0;
-    for (int i = threadIdx.x; i < nblocks; i += blockDim.x) acc += partial[rhs * nblocks + i];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[rhs] = 0.5 * red[0];
-}
-
-int device_energy(Mesh& m, const void* state, double* out_host, void* stream) {
-    MTP_TRY(device_mesh_upload(m));
-    cudaStream_t st = (cudaStream_t)stream;
-    dim3 grid(kEnergyBlocks, m.n_rhs);
-    if (state_f64(m))
-        energy_partial_kernel<double><<<grid, kEnergyThreads, 0, st>>>((const double*)state, m.dev->geo, m.ne, m.nf,
-                                                                        m.nb, m.dev->partial);
-    else
-        energy_partial_kernel<float><<<grid, kEnergyThreads, 0, st>>>((const float*)state, m.dev->geo, m.ne, m.nf,
-                                                                       m.nb, m.dev->partial);
-    CUDA_TRY(cudaGetLastError());
-    double* out_dev = m.dev->partial + (size_t)kEnergyBlocks * m.n_rhs;
-    energy_final_kernel<<<m.n_rhs, kEnergyThreads, 0, st>>>(m.dev->partial, kEnergyBlocks, out_dev);
-    CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(cudaMemcpyAsync(out_host, out_dev, sizeof(double) * m.n_rhs, cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
-    return MTP_OK;
-}
+const double* device_geo(const Mesh& m) { return m.dev->geo; }
+double* device_energy_scratch(const Mesh& m) { return m.dev->partial; }
 
 // ---------------------------------------------------------------------------------
 // evolution

@@ -1,6 +1,7 @@
-"""Apex tent kernel (3D, p = 1..4) and its many-instance form at the sizes where they can go wrong:
-patches from 1 to 24 elements, every local index of the tent vertex and both element
-orientations (shuffled vertex numbers), material jumps in eps and mu, several right-hand sides.
+"""Apex tent kernel (3D, p = 1..4), its many-instance form, and the lattice / energy kernels at the
+sizes where they can go wrong: patches from 1 to 24 elements, every local index of the tent
+vertex and both element orientations (shuffled vertex numbers), material jumps in eps and mu,
+several right-hand sides, element counts around the 32 of a block.
 
 Tolerances: those of the precision contract (FP64 1e-11, FP32 1e-5 against the oracle);
 the two launch configurations run the same device code on the same inputs, so equality is asked."""
@@ -83,3 +84,28 @@ def test_apex_batch_of_all_degrees_equals_single_evolves():
             # one set of device functions compiled into two kernels: equal up to contraction choices
             for a, b in zip(states, ref):
                 assert rel_l2(a.cpu().numpy(), b.cpu().numpy()) <= (1e-13 if prec == mtp.MTP_FP64 else 1e-6)
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5])
+def test_lattice_exchange_and_energy(dim, p):
+    """Element counts 1, 31 .. 33 of a longer mesh; values against the oracle's energy and the exact roundtrip."""
+    full_v, full_e = S.square_mesh(5) if dim == 2 else S.cube_mesh(2)
+    rng = np.random.default_rng(p)
+    for ne in (1, 31, 32, 33):
+        e = full_e[:ne]
+        used = np.unique(e)
+        back = np.full(len(full_v), -1)
+        back[used] = np.arange(len(used))
+        v, e = full_v[used], back[e].astype(np.int32)
+        eps, mu = rng.uniform(1, 3, ne), rng.uniform(1, 2, ne)
+        nf, nb = (3, (p + 1) * (p + 2) // 2) if dim == 2 else (6, (p + 1) * (p + 2) * (p + 3) // 6)
+        vals = rng.standard_normal((2, ne, nb, nf))
+        disc = Discretization(OMesh(v, e, eps, mu), p)
+        want = [disc.energy(disc.fields_at_flat_front(disc.moments_from_lattice(x))) for x in vals]
+        for prec, tol in ((mtp.MTP_FP64, 1e-11), (mtp.MTP_FP32, 1e-5)):
+            mesh = mtp.Mesh(dim, v, e, eps, mu, p=p, precision=prec, n_rhs=2)
+            st = mesh.state_from_lattice(torch.tensor(vals, device=DEV))
+            out = mesh.state_to_lattice(st).cpu().numpy()
+            assert rel_l2(out, vals) <= tol and max_rel(out, vals) <= tol
+            assert np.allclose(mesh.energy(st), want, rtol=tol, atol=0)
