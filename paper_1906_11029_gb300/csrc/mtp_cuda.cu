@@ -1,4 +1,5 @@
 // Device-side management of the MTP library: uploads and the evolution drivers.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -8,6 +9,7 @@
 
 #include "mtp_adjoint.cuh"
 #include "mtp_apex.cuh"
+#include "mtp_apex2.cuh"
 #include "mtp_device.h"
 #include "mtp_internal.h"
 #include "mtp_launch.cuh"
@@ -41,6 +43,7 @@ struct DeviceMesh {
     float* Dtc = nullptr;         // tcgen05 A operand (variants 3, 4): D^T in core-matrix layout, hi then lo
     void* ent = nullptr;          // apex tent kernel: patch entry records, change of basis
     void* Rt = nullptr;
+    void* apex2 = nullptr;        // tables of the 2D apex tent kernel
     double* partial = nullptr;    // energy reduction scratch: [n_rhs][kEnergyBlocks] partials, then [n_rhs] sums
 };
 
@@ -234,9 +237,121 @@ static int apex_upload_real(const Mesh& m, DeviceMesh& d) {
     return MTP_OK;
 }
 
-// the apex tent kernel runs the plain SAT modes in 3D up to kApexMaxDegree
+// the same in 2D (layout at kApex2Rec); one thread per patch entry
+template <typename Real>
+__global__ void apex2_record_kernel(int64_t nv, const int64_t* patch_ptr, const int32_t* patch_elem,
+                                    const int8_t* patch_info, const double* geo, Real* ent) {
+    const int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+    if (v >= nv) return;
+    const int64_t pb = patch_ptr[v];
+    for (int64_t at = pb + (threadIdx.x & 15); at < patch_ptr[v + 1]; at += 16) {
+        const int8_t* info = patch_info + at * 12;
+        const double* g = geo + (int64_t)patch_elem[at] * kGeoStride;
+        const int j = info[0];
+        double gr[2][2], t[2][2];
+        for (int w = 0; w < 2; ++w)
+            for (int q = 0; q < 2; ++q) gr[w][q] = g[3 * (w < j ? w : w + 1) + q];
+        const double dg = gr[0][0] * gr[1][1] - gr[0][1] * gr[1][0];
+        const double s = g[28], l = exp2(rint(log2(1.0 / (s * s)) / 2.0));
+        t[0][0] = gr[1][1] / dg / l;
+        t[0][1] = -gr[1][0] / dg / l;
+        t[1][0] = -gr[0][1] / dg / l;
+        t[1][1] = gr[0][0] / dg / l;
+        for (int w = 0; w < 2; ++w)
+            for (int q = 0; q < 2; ++q) gr[w][q] *= l;
+        const double det = 1.0 / (dg * l * l), sgn = det > 0 ? 1.0 : -1.0, c1 = 1.0 / (l * det), eps = g[29], mu = g[30];
+        Real* r = ent + at * kApex2Rec;
+        auto dot = [](const double* x, const double* y) { return x[0] * y[0] + x[1] * y[1]; };
+        r[0] = (Real)dot(t[0], t[0]);
+        r[1] = (Real)dot(t[0], t[1]);
+        r[2] = (Real)dot(t[1], t[1]);
+        r[3] = (Real)dot(gr[0], gr[0]);
+        r[4] = (Real)dot(gr[0], gr[1]);
+        r[5] = (Real)dot(gr[1], gr[1]);
+        r[6] = (Real)(1.0 / l);
+        r[7] = (Real)eps;
+        r[8] = (Real)mu;
+        r[9] = (Real)(c1 / (l * s));
+        r[10] = (Real)(1.0 / (eps * mu));
+        r[11] = (Real)c1;
+        r[12] = (Real)(-s / c1);
+        r[13] = (Real)(l * s / c1);
+        r[14] = (Real)(1.0 / det);
+        for (int f = 0; f < 2; ++f) {
+            const int s2 = info[4 + (1 - f < j ? 1 - f : 2 - f)];
+            const double zm = g[31], zp = s2 >= 0 ? geo[(int64_t)patch_elem[pb + s2] * kGeoStride + 31] : zm;
+            const double len = l * sqrt(dot(t[f], t[f]));
+            r[15 + 4 * f] = (Real)(zm / (zm + zp));
+            r[16 + 4 * f] = (Real)(zp / (zm + zp));
+            r[17 + 4 * f] = (Real)(sgn / (len * (zm + zp)));
+            r[18 + 4 * f] = (Real)(sgn * zm * zp * len / (zm + zp));
+        }
+        for (int w = 0; w < 2; ++w)
+            for (int q = 0; q < 2; ++q) {
+                r[23 + 2 * w + q] = (Real)gr[w][q];
+                r[27 + 2 * w + q] = (Real)t[w][q];
+            }
+        r[31] = (Real)(-c1 / s);
+    }
+}
+
+template <typename Real>
+static int apex2_upload_real(const Mesh& m, DeviceMesh& d) {
+    const RefTables& r = m.ref;
+    const int nb = m.nb, nfb = m.nfb;
+    std::vector<Real> t((size_t)nb * nb, Real(0));
+    std::vector<uint8_t> rows(4 * nb + nb * nb + nb, 0);
+    auto parity = [](int b) {
+        int g = 0;
+        while (b >= (g + 1) * (g + 2) / 2) ++g;
+        return (b - g * (g + 1) / 2) & 1;
+    };
+    int n = 0;
+    for (int a = 0; a < nb; ++a) {   // compressed rows: equal parity first
+        rows[4 * a] = (uint8_t)(n & 255);
+        rows[4 * a + 1] = (uint8_t)(n >> 8);
+        for (int opp = 0; opp < 2; ++opp)
+            for (int b = 0; b < nb; ++b)
+                if ((parity(a) != parity(b)) == (opp == 1) && r.C2[(size_t)a * nb + b] != 0.0) {
+                    t[n] = (Real)r.C2[(size_t)a * nb + b];
+                    rows[4 * nb + n] = (uint8_t)b;
+                    rows[4 * a + 2 + opp]++;
+                    ++n;
+                }
+        if (rows[4 * a + 2] + rows[4 * a + 3] > kApex2MaxRow[m.p - 1])
+            return set_error(MTP_EINVAL, "2D apex tables: a row is longer than the kernel reads");
+        rows[4 * nb + nb * nb + a] = (uint8_t)a;
+    }
+    std::stable_sort(rows.end() - nb, rows.end(), [&](uint8_t a, uint8_t b) {
+        return rows[4 * a + 2] + rows[4 * a + 3] < rows[4 * b + 2] + rows[4 * b + 3];
+    });
+    for (double v : r.T2) t.push_back((Real)v);
+    for (double v : r.L2) t.push_back((Real)v);
+    for (int j = 0; j < 3; ++j)
+        for (int a = 0, g = 0; a < nb; ++a) {
+            while (a >= (g + 1) * (g + 2) / 2) ++g;
+            for (int b = 0; b < nfb; ++b)
+                t.push_back(b <= g ? (Real)r.Rot[((size_t)j * nb + a) * nb + g * (g + 1) / 2 + b] : Real(0));
+        }
+    std::vector<uint8_t> buf(t.size() * sizeof(Real) + rows.size());
+    std::memcpy(buf.data(), t.data(), t.size() * sizeof(Real));
+    std::memcpy(buf.data() + t.size() * sizeof(Real), rows.data(), rows.size());
+    MTP_TRY(upload((uint8_t**)&d.apex2, buf.data(), buf.size()));
+    CUDA_TRY(cudaMalloc(&d.ent, m.patch_elem.size() * kApex2Rec * sizeof(Real) + 16));
+    const int64_t blocks = (m.nv * 16 + 127) / 128;
+    apex2_record_kernel<Real><<<(unsigned)blocks, 128>>>(m.nv, d.patch_ptr, d.patch_elem, d.patch_info, d.geo, (Real*)d.ent);
+    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(cudaDeviceSynchronize());
+    return MTP_OK;
+}
+
+// the apex tent kernels run the plain SAT modes in 2D, and in 3D up to kApexMaxDegree
 static int apex_upload(const Mesh& m, DeviceMesh& d) {
-    if (m.dim != 3 || m.p > kApexMaxDegree) return MTP_OK;
+    if (m.dim == 2) {
+        if (m.precision == MTP_FP64) return apex2_upload_real<double>(m, d);
+        return m.precision == MTP_FP32 ? apex2_upload_real<float>(m, d) : MTP_OK;
+    }
+    if (m.p > kApexMaxDegree) return MTP_OK;
     if (m.precision == MTP_FP64) return apex_upload_real<double>(m, d);
     return m.precision == MTP_FP32 ? apex_upload_real<float>(m, d) : MTP_OK;
 }
@@ -333,7 +448,7 @@ void device_mesh_free(Mesh& m) {
     DeviceMesh& d = *m.dev;
     void* ptrs[] = {d.geo, d.elems, d.patch_ptr, d.patch_elem, d.patch_info, d.S, d.Tr, d.L, d.Mc, d.Dc, d.Trc, d.Lc, d.Mc1, d.Dc1, d.Trc1, d.Lc1,
                     d.partial,
-                    d.Sf, d.Lfr, d.Trf, d.Sf_lo, d.Lfr_lo, d.Trf_lo, d.Dtc, d.ent, d.Rt};
+                    d.Sf, d.Lfr, d.Trf, d.Sf_lo, d.Lfr_lo, d.Trf_lo, d.Dtc, d.ent, d.Rt, d.apex2};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete m.dev;
@@ -456,6 +571,7 @@ static void fill_args(Tents& t, void* state, KArgs& a) {
     a.Dtc = dm.Dtc;
     a.ent = dm.ent;
     a.Rt = dm.Rt;
+    a.apex2 = dm.apex2;
     a.state = state;
     a.rhs_stride = m.ne * m.nf * m.nb;
     a.err = dt.err;
@@ -790,7 +906,7 @@ int device_batch_evolve(Batch& b, void* const* states, void* stream) {
     const int64_t ni = (int64_t)b.inst.size();
     for (Tents* t : b.inst) MTP_TRY(device_tents_upload(*t));
     const Mesh& m0 = *b.inst[0]->mesh;
-    static BatchEntry table[2][2];
+    static BatchEntry table[2];
     static bool init = false;
     if (!init) { batch_table(table); init = true; }
     for (Tents* t : b.inst)
@@ -800,8 +916,10 @@ int device_batch_evolve(Batch& b, void* const* states, void* stream) {
         return set_error(MTP_EUNSUPPORTED, "batches run FP64 or FP32 SIMT meshes; tensor-core and split modes are per mesh");
     int pmax = 0;
     for (Tents* t : b.inst) pmax = std::max(pmax, t->mesh->p);
-    BatchEntry be = table[m0.precision == MTP_FP64 ? 0 : 1][m0.dim - 2];
-    if (m0.dim == 3 && pmax <= kApexMaxDegree) be = m0.precision == MTP_FP64 ? apex_batch_f64(pmax) : apex_batch_f32(pmax);
+    const bool f64 = m0.precision == MTP_FP64;
+    const BatchEntry be = m0.dim == 2              ? (f64 ? apex2_batch_f64() : apex2_batch_f32())
+                          : pmax <= kApexMaxDegree ? (f64 ? apex_batch_f64(pmax) : apex_batch_f32(pmax))
+                                                   : table[f64 ? 0 : 1];
     if (!b.dev) {
         b.dev = new DeviceBatch();
         DeviceBatch& d = *b.dev;

@@ -36,10 +36,17 @@ struct RefTables {
     std::vector<double> Tr;
     // L[j][f][a][c] = int_{F^} lambda_j(x_f(s)) psi_a(x_f(s)) chi_c(s) ds
     std::vector<double> L;
-    // 3D, p <= kApexMaxDegree: Rot[j][a][b] = int psi'_a psi_b with psi' the basis on the element
-    // whose collapsed apex is local vertex j (coordinates: the other vertices in ascending order
-    // take the places C, D, B of the apex tent kernel); orthogonal, block-diagonal in the degree
+    // 2D, and 3D with p <= kApexMaxDegree: Rot[j][a][b] = int psi'_a psi_b with psi' the basis on
+    // the element whose collapsed apex is local vertex j (coordinates: the other vertices in ascending
+    // order take the places C, D and, in 3D, B of the apex tent kernels); orthogonal,
+    // block-diagonal in the degree
     std::vector<double> Rot;
+    // 2D apex tent kernel (V at y = 1, edges to C = origin and D): with S_X[a][b] = int psi_b lambda_V
+    // (derivative of psi_a along the edge to X), C2[a][b] = (S_C + S_D) / 2 where the collapsed indices
+    // of a and b have equal parity and (S_D - S_C) / 2 elsewhere (the other entries vanish);
+    // T2[n][a] and L2[a][n] the trace on and the lambda_V-weighted lift from the edge to C (odd
+    // functions change sign on the other edge)
+    std::vector<double> C2, T2, L2;
     // V[k][a] = psi_a(lattice point k), Vinv its inverse
     std::vector<double> V, Vinv;
     double max_orth_err = 0;   // max |int psi_a psi_b - delta_ab| (diagnostic)

@@ -72,6 +72,7 @@ struct KArgs {
     // the change of basis per local index of V
     const void* ent;
     const void* Rt;
+    const void* apex2;          // 2D: tables of the 2D apex tent kernel (mtp_apex2.cuh)
     void* state;                // [rhs][ne][nf][nb]
     int64_t rhs_stride;         // ne * nf * nb
     int* err;                   // error word (0 = ok, 1 = causality, 2 = non-finite)

@@ -84,6 +84,9 @@ void kernel_table_f32_tc5(KernelEntry entries[2][5]);
 // apex tent kernel, 3D, p <= kApexMaxDegree (mtp_apex.cuh)
 KernelEntry apex_entry_f32(int p);
 KernelEntry apex_entry_f64(int p);
+// 2D, p = 1..5 (mtp_apex2.cuh)
+KernelEntry apex2_entry_f32(int p);
+KernelEntry apex2_entry_f64(int p);
 
 struct AdjArgs;
 using AdjLaunchFn = cudaError_t (*)(const AdjArgs&, int64_t t0, int n_tents, int n_rhs, cudaStream_t st);
@@ -104,11 +107,14 @@ struct BatchEntry {
     BatchPrepFn prepare;
     BatchSmemFn smem_bytes;
 };
-// entries[precision][dim - 2]
-void batch_table(BatchEntry entries[2][2]);
+// 3D batches with degrees beyond the apex kernel's: entries[precision]
+void batch_table(BatchEntry entries[2]);
 // 3D batches whose largest degree is at most kApexMaxDegree
 BatchEntry apex_batch_f32(int pmax);
 BatchEntry apex_batch_f64(int pmax);
+// 2D batches
+BatchEntry apex2_batch_f32();
+BatchEntry apex2_batch_f64();
 
 #define MTP_KERNEL_ENTRY(REAL, D, P, MODE)                                                      \
     KernelEntry{launch_tent_kernel<REAL, D, P, MODE>, prepare_tent_kernel<REAL, D, P, MODE>,     \

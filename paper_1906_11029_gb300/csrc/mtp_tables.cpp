@@ -355,13 +355,44 @@ RefTables build_ref_tables(int d, int p) {
                     if (!(std::fabs((double)acc - t.S[(((size_t)j * d + l) * nb + a) * nb + b]) <= 1e-12 * smax))
                         throw std::runtime_error("reference tables: factored volume tables do not reproduce S");
                 }
-    if (d == 3 && p <= kApexMaxDegree) {
+    if (d == 2) {
+        const Poly X = Poly::var(0), Y = Poly::var(1), zero_p;
+        auto along = [&](int a, ld dx, ld dy) { return add(scale(deriv(psi[a], 0), dx), scale(deriv(psi[a], 1), dy)); };
+        std::vector<int> par(nb);
+        for (int a = 0, g = 0; a < nb; ++a) {
+            while (a >= (g + 1) * (g + 2) / 2) ++g;
+            par[a] = (a - g * (g + 1) / 2) & 1;
+        }
+        t.C2.assign((size_t)nb * nb, 0.0);
+        for (int a = 0; a < nb; ++a)
+            for (int b = 0; b < nb; ++b) {
+                const Poly yb = mul(Y, psi[b]);
+                double same = (double)integrate(mul(yb, along(a, 0.5L, -1)), 2), opp = (double)integrate(mul(yb, along(a, 0.5L, 0)), 2);
+                zero(par[a] == par[b] ? opp : same, 1.0);
+                const double v = par[a] == par[b] ? same : opp;
+                t.C2[(size_t)a * nb + b] = std::fabs(v) < 1e-14 ? 0.0 : v;
+            }
+        t.T2.assign((size_t)nfb * nb, 0.0);
+        t.L2.assign((size_t)nb * nfb, 0.0);
+        for (int a = 0; a < nb; ++a) {
+            const Poly c0 = compose(psi[a], zero_p, X, zero_p), c1 = compose(psi[a], add(Poly::cst(1), X, -1), X, zero_p);
+            for (int n = 0; n < nfb; ++n) {
+                t.T2[(size_t)n * nb + a] = (double)integrate(mul(chi[n], c0), 1);
+                t.L2[(size_t)a * nfb + n] = (double)integrate(mul(mul(X, c0), chi[n]), 1);
+                double mirror = (double)integrate(mul(chi[n], c1), 1) - (par[a] ? -1 : 1) * t.T2[(size_t)n * nb + a];
+                zero(mirror, 1.0);
+                if (dchi_deg[n] > dpsi_deg[a]) zero(t.T2[(size_t)n * nb + a], 1.0);
+            }
+        }
+    }
+    if (d == 2 || p <= kApexMaxDegree) {
         t.Rot.assign((size_t)(d + 1) * nb * nb, 0.0);
         for (int j = 0; j <= d; ++j) {
-            std::vector<Poly> at;   // coordinates x, y, z of the apex frame: lambda_D, lambda_B, lambda_A
+            std::vector<Poly> at;   // coordinates of the apex frame: lambda_D, lambda_B, lambda_A (2D: lambda_D, lambda_A)
             for (int i = 0, n = 0; i <= d; ++i)
                 if (i != j && n++ > 0) at.push_back(lam[i]);
             at.push_back(lam[j]);
+            at.resize(3);           // z = 0 in 2D
             for (int a = 0; a < nb; ++a) {
                 const Poly r = compose(psi[a], at[0], at[1], at[2]);
                 for (int b = 0; b < nb; ++b) {

@@ -1,7 +1,8 @@
-"""Apex tent kernel (3D, p = 1..4), its many-instance form, and the lattice / energy kernels at the
-sizes where they can go wrong: patches from 1 to 24 elements, every local index of the tent
-vertex and both element orientations (shuffled vertex numbers), material jumps in eps and mu,
-several right-hand sides, element counts around the 32 of a block.
+"""Apex tent kernels (3D, p = 1..4; 2D, p = 1..5), their many-instance forms, and the lattice / energy
+kernels at the sizes where they can go wrong: patches from one element to the most that is accepted
+(32 in 3D, 16 in 2D), every local index of the tent vertex and both element orientations (shuffled
+vertex numbers), material jumps in eps and mu, several right-hand sides, element counts around the
+32 of a block.
 
 Tolerances: those of the precision contract (FP64 1e-11, FP32 1e-5 against the oracle);
 the two launch configurations run the same device code on the same inputs, so equality is asked."""
@@ -27,7 +28,32 @@ TOL = {mtp.MTP_FP64: 1e-11, mtp.MTP_FP32: 1e-5}
 def _problem(name, seed=3):
     """(verts, elems, eps, mu): shuffled vertex numbers put the tent vertex at every local index."""
     rng = np.random.default_rng(seed)
-    if name == "one_tet":
+    if name == "one_tri":
+        v, e = np.array([[0., 0], [1, .1], [.3, .8]]), np.array([[0, 1, 2]], np.int32)
+    elif name in ("square1", "square3"):
+        v, e = S.square_mesh(int(name[-1]))
+        v = S.perturb_interior(v, 1.0 / 3, 0.15, 7)
+    elif name == "fan16":
+        t = 2 * np.pi * np.arange(16) / 16
+        v = np.concatenate([[[0.0, 0.0]], np.stack([np.cos(t), np.sin(t)], 1)])
+        e = np.array([[0, 1 + i, 1 + (i + 1) % 16] for i in range(16)], np.int32)
+    elif name == "ball32":   # octahedron with every face split in four, coned from its centre
+        v = [np.zeros(3)] + [s * x for x in np.eye(3) for s in (1.0, -1.0)]
+        mid, e = {}, []
+
+        def middle(a, b):
+            if (min(a, b), max(a, b)) not in mid:
+                mid[(min(a, b), max(a, b))] = len(v)
+                v.append((v[a] + v[b]) / np.linalg.norm(v[a] + v[b]))
+            return mid[(min(a, b), max(a, b))]
+
+        for a in (1, 2):
+            for b in (3, 4):
+                for c in (5, 6):
+                    ab, bc, ca = middle(a, b), middle(b, c), middle(c, a)
+                    e += [[0, a, ab, ca], [0, b, ab, bc], [0, c, bc, ca], [0, ab, bc, ca]]
+        v, e = np.array(v), np.array(e, np.int32)
+    elif name == "one_tet":
         v, e = np.array([[0., 0, 0], [1, .1, 0], [.2, .9, .1], [.1, .3, 1.1]]), np.array([[0, 1, 2, 3]], np.int32)
     else:
         n = {"cube1": 1, "cube2": 2, "graded3": 3}[name]
@@ -47,14 +73,20 @@ def _oracle(v, e, eps, mu, p, T, vals):
     return disc.eval_lattice(disc.y_coeffs(Y))
 
 
-@pytest.mark.parametrize("p", [1, 2, 3, 4])
-@pytest.mark.parametrize("name,T", [("one_tet", 0.1), ("cube1", 0.1), ("cube2", 0.05), ("graded3", 0.02)])
+_CASES = [(n, T, p) for n, T in (("one_tet", 0.1), ("cube1", 0.1), ("cube2", 0.05), ("graded3", 0.02), ("ball32", 0.06))
+          for p in (1, 2, 3, 4)]
+_CASES += [(n, T, p) for n, T in (("one_tri", 0.2), ("square1", 0.2), ("square3", 0.1), ("fan16", 0.1)) for p in (1, 2, 3, 4, 5)]
+
+
+@pytest.mark.parametrize("name,T,p", _CASES)
 def test_apex_kernel_matches_oracle(name, T, p):
     v, e, eps, mu = _problem(name)
-    vals = np.random.default_rng(p).standard_normal((len(e), (p + 1) * (p + 2) * (p + 3) // 6, 6))
+    dim = v.shape[1]
+    nf, nb = (3, (p + 1) * (p + 2) // 2) if dim == 2 else (6, (p + 1) * (p + 2) * (p + 3) // 6)
+    vals = np.random.default_rng(p).standard_normal((len(e), nb, nf))
     ref = _oracle(v, e, eps, mu, p, T, vals)
     for prec in (mtp.MTP_FP64, mtp.MTP_FP32):
-        mesh = mtp.Mesh(3, v, e, eps, mu, p=p, precision=prec, n_rhs=2)
+        mesh = mtp.Mesh(dim, v, e, eps, mu, p=p, precision=prec, n_rhs=2)
         tents = mesh.pitch(T, 0.5)
         outs = []
         for launch in (0, 2):
@@ -68,22 +100,25 @@ def test_apex_kernel_matches_oracle(name, T, p):
         assert torch.equal(outs[0], outs[1])
 
 
-def test_apex_batch_of_all_degrees_equals_single_evolves():
-    v, e, eps, mu = _problem("cube2")
+@pytest.mark.parametrize("name,degrees", [("cube2", (1, 2)), ("cube2", (3, 1, 2)), ("cube2", (4, 2, 3, 1)), ("cube2", (5, 2)),
+                                          ("square3", (5, 1, 3)), ("square3", (4, 2))])
+def test_batch_of_all_degrees_equals_single_evolves(name, degrees):
+    v, e, eps, mu = _problem(name)
     for prec in (mtp.MTP_FP64, mtp.MTP_FP32):
-        for degrees in ((1, 2), (3, 1, 2), (4, 2, 3, 1)):
-            tents, states, ref = [], [], []
-            for i, p in enumerate(degrees):
-                mesh = mtp.Mesh(3, v, e, eps, mu, p=p, precision=prec, n_rhs=1 + i % 2)
-                tents.append(mesh.pitch(0.04, 0.5))
-                st = torch.randn(mesh.state_shape, generator=torch.Generator().manual_seed(i), dtype=torch.float64)
-                states.append(st.to(DEV, mesh.torch_dtype()))
-                ref.append(states[-1].clone())
-                tents[-1].evolve(ref[-1])
-            mtp.Batch(tents).evolve(states)
-            # one set of device functions compiled into two kernels: equal up to contraction choices
-            for a, b in zip(states, ref):
-                assert rel_l2(a.cpu().numpy(), b.cpu().numpy()) <= (1e-13 if prec == mtp.MTP_FP64 else 1e-6)
+        if prec == mtp.MTP_FP64 and name == "cube2" and max(degrees) == 5:
+            continue    # FP64 p = 5 in 3D needs more shared memory than a block may have
+        tents, states, ref = [], [], []
+        for i, p in enumerate(degrees):
+            mesh = mtp.Mesh(v.shape[1], v, e, eps, mu, p=p, precision=prec, n_rhs=1 + i % 2)
+            tents.append(mesh.pitch(0.04, 0.5))
+            st = torch.randn(mesh.state_shape, generator=torch.Generator().manual_seed(i), dtype=torch.float64)
+            states.append(st.to(DEV, mesh.torch_dtype()))
+            ref.append(states[-1].clone())
+            tents[-1].evolve(ref[-1])
+        mtp.Batch(tents).evolve(states)
+        # FP64: the same arithmetic compiled into another kernel; FP32 batches with p = 5 run the general one
+        for a, b in zip(states, ref):
+            assert rel_l2(a.cpu().numpy(), b.cpu().numpy()) <= (1e-13 if prec == mtp.MTP_FP64 else 1e-5)
 
 
 @pytest.mark.parametrize("dim", [2, 3])
@@ -109,3 +144,22 @@ def test_lattice_exchange_and_energy(dim, p):
             out = mesh.state_to_lattice(st).cpu().numpy()
             assert rel_l2(out, vals) <= tol and max_rel(out, vals) <= tol
             assert np.allclose(mesh.energy(st), want, rtol=tol, atol=0)
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_vertex_without_elements(dim):
+    """A vertex that no element uses has a tent of no elements; the rest of the mesh is not affected."""
+    v, e = S.square_mesh(2) if dim == 2 else S.cube_mesh(1)
+    one = np.ones(len(e))
+    outs = []
+    for extra in (0, 1):
+        vv = np.concatenate([v, np.full((extra, dim), 5.0)])
+        mesh = mtp.Mesh(dim, vv, e, one, one, p=2, precision=mtp.MTP_FP64)
+        tents = mesh.pitch(0.1, 0.5)
+        assert len(tents.get()["vertex"]) == len(mesh.pitch(0.1, 0.5, device=True).get()["vertex"])
+        for launch in (0, 2):
+            tents.set_launch(launch)
+            st = torch.ones(mesh.state_shape, dtype=torch.float64, device=DEV)
+            tents.evolve(st)
+            outs.append(st)
+    assert all(torch.equal(outs[0], o) for o in outs[1:])
