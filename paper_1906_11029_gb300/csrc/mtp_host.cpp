@@ -302,45 +302,24 @@ int pitch_graph(const Mesh& m, const double* wavespeed, double cf, PitchGraph& g
         }
         for (int i = 0; i < nvert; ++i) k[el[i]] = std::fmin(k[el[i]], H[i]);
     }
-    // edges: (a < b) -> max wave speed; then directed CSR sorted by (src, dst)
-    std::vector<std::pair<int64_t, double>> ekeys;   // key = a * nv + b
-    ekeys.reserve(ne * nvert * d / 2);
-    for (int64_t e = 0; e < ne; ++e) {
-        const int32_t* el = &m.elems[e * nvert];
-        for (int i = 0; i < nvert; ++i)
-            for (int j = i + 1; j < nvert; ++j) ekeys.emplace_back((int64_t)el[i] * nv + el[j], c[e]);
-    }
-    std::sort(ekeys.begin(), ekeys.end());
-    std::vector<int64_t>& ptr = g.ptr;
-    ptr.assign(nv + 1, 0);
-    std::vector<std::pair<int64_t, double>> edges;   // unique, with max c
-    for (size_t i = 0; i < ekeys.size();) {
-        size_t j = i;
-        double cm = ekeys[i].second;
-        while (j < ekeys.size() && ekeys[j].first == ekeys[i].first) { cm = std::fmax(cm, ekeys[j].second); ++j; }
-        edges.emplace_back(ekeys[i].first, cm);
-        i = j;
-    }
-    for (auto& ed : edges) { ptr[ed.first / nv + 1]++; ptr[ed.first % nv + 1]++; }
-    for (int64_t v = 0; v < nv; ++v) ptr[v + 1] += ptr[v];
-    std::vector<int32_t>& dst = g.dst;
-    std::vector<double>& bnd = g.bnd;
-    dst.assign(ptr[nv], 0);
-    bnd.assign(ptr[nv], 0.0);
-    {
-        std::vector<int64_t> fill(ptr.begin(), ptr.end() - 1);
-        for (auto& ed : edges) {
-            int64_t a = ed.first / nv, b = ed.first % nv;
-            double bab = (cf * std::fmin(k[a], k[b])) / ((double)d * ed.second);
-            dst[fill[a]] = (int32_t)b; bnd[fill[a]++] = bab;
-            dst[fill[b]] = (int32_t)a; bnd[fill[b]++] = bab;
+    // directed edges in the order of the mesh's adjacency (rows ascending), largest wave speed of the
+    // elements at the edge
+    g.ptr.assign(m.adj_ptr.begin(), m.adj_ptr.end());
+    g.dst.assign(m.adj.begin(), m.adj.end());
+    g.bnd.assign(g.dst.size(), 0.0);
+    for (int64_t v = 0; v < nv; ++v) {
+        const int32_t *row = g.dst.data() + g.ptr[v], *end = g.dst.data() + g.ptr[v + 1];
+        double* cm = g.bnd.data() + g.ptr[v];
+        for (int64_t q = m.patch_ptr[v]; q < m.patch_ptr[v + 1]; ++q) {
+            const int32_t e = m.patch_elem[q];
+            for (int i = 0; i < nvert; ++i) {
+                const int32_t w = m.elems[(int64_t)e * nvert + i];
+                if (w == v) continue;
+                double& x = cm[std::lower_bound(row, end, w) - row];
+                x = std::fmax(x, c[e]);
+            }
         }
-        for (int64_t v = 0; v < nv; ++v) {   // sort each row by dst
-            std::vector<std::pair<int32_t, double>> row;
-            for (int64_t q = ptr[v]; q < ptr[v + 1]; ++q) row.emplace_back(dst[q], bnd[q]);
-            std::sort(row.begin(), row.end());
-            for (int64_t q = ptr[v]; q < ptr[v + 1]; ++q) { dst[q] = row[q - ptr[v]].first; bnd[q] = row[q - ptr[v]].second; }
-        }
+        for (int64_t q = 0; q < end - row; ++q) cm[q] = (cf * std::fmin(k[v], k[row[q]])) / ((double)d * cm[q]);
     }
     return MTP_OK;
 }

@@ -1,23 +1,20 @@
 // Tent pitching on the GPU (mtp_pitch_tents_device, see include/mtp.h): the same rounds and
 // the same FP64 arithmetic as the host pitcher, so the tent list is bit-identical.
 //
-// One round (Sec. 2: vertices that are not neighbours may be advanced independently):
-//   select: every vertex V with tau_V < T that is a strict local minimum of (tau, id) over
-//           its neighbours gets tau'_V = min(T, min_W tau_W + b_VW) and
-//           layer_V = 1 + max(last_V, last_W), all from the values at the start of the round;
-//   scan:   one block prefix-sums the per-block counts of selected vertices and commits the
-//           round (or stops: nothing selected, or the output arrays are full);
-//   emit:   the selected vertices write their tents in ascending vertex order and apply
-//           tau'_V, layer_V.
-// Selected vertices are never neighbours of each other, so select reads only values that
-// no thread of the same round changes before emit runs.
+// A round (Sec. 2: vertices that are not neighbours may be advanced independently) selects every
+// vertex V with tau_V < T that is a strict local minimum of (tau, id) over its neighbours and moves
+// it to tau'_V = min(T, min_W tau_W + b_VW), all from the values at the start of the round.  There are
+// thousands of rounds with little work each, so they run inside one cooperative kernel: a block
+// owns a contiguous range of vertices, tau is double-buffered by the round's parity, and one grid
+// barrier ends a round (its last arriver decides whether the rounds go on).  A block appends its
+// tents to a list of its own; after kPitchChunk rounds two kernels order the lists by (round,
+// block), which is (round, vertex) since blocks own ascending ranges.  (Three kernels a round
+// took 37 us a round on a mesh of 4913 vertices, launches and their gaps for the most part.)
 //
-// Layer = round: if V is selected in round r and no vertex of {V} u N(V) moved in round
-// r - 1, V's test gave the same answer in round r - 1 and V would have moved then; so some
-// vertex of the closed neighbourhood has last = r - 1 and layer_V = r (by induction, no
-// last exceeds r - 1). Emitting each round in vertex order therefore produces the list
-// sorted by (layer, vertex) without a sort; emit checks layer == round and reports an
-// internal error otherwise.
+// Layer = round: if V is selected in round r and no vertex of {V} u N(V) moved in round r - 1, V's
+// test gave the same answer in round r - 1 and V would have moved then; so some vertex of the closed
+// neighbourhood moved in round r - 1 and layer_V = 1 + max(last layers) = r by induction.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -29,136 +26,182 @@
 
 namespace mtp {
 
-constexpr int kPitchThreads = 1024;   // vertices per block (select / emit) and scan width
-constexpr int kPitchRoundsPerSync = 32;
-constexpr int kPitchMaxRounds = 50000000;
+constexpr int kPitchThreads = 256;
+constexpr int kPitchChunk = 128;              // rounds per launch at most
+constexpr long long kPitchMaxRounds = 50000000;
 
 struct PitchCtl {
-    long long count;      // tents committed
-    long long capacity;   // tent capacity of the output arrays
-    long long base;       // first tent of the round being emitted
-    int round;            // next round to run
-    int cur;              // round being emitted
-    int layer_cap;        // capacity of layer_ptr (entries after the first)
-    int stop;             // 0 running, 1 finished (a round selected nothing), 2 out of capacity
-    int err;              // 1: a tent's layer differs from its round
+    unsigned arrived;           // blocks that reached the barrier, over the whole launch
+    unsigned released;          // rounds whose barrier is open
+    int selected;               // vertices selected in the round
+    int left;                   // vertices with tau < T
+    int stop;                   // 1 all at T, 2 a round selected nothing, 3 a barrier wait expired
+    int rounds;                 // rounds done by the launch
 };
 
-__global__ void __launch_bounds__(kPitchThreads) pitch_select_kernel(
-    const PitchCtl* ctl, int64_t nv, double T, const int64_t* ptr, const int32_t* dst, const double* bnd,
-    const double* tau, const int32_t* last, uint8_t* flag, double* newt, int32_t* newl, int* blockcnt) {
-    if (ctl->stop) return;
-    const int64_t v = (int64_t)blockIdx.x * kPitchThreads + threadIdx.x;
-    int sel = 0;
-    if (v < nv) {
-        const double tv = tau[v];
-        if (tv < T) {
-            sel = 1;
-            for (int64_t q = ptr[v]; q < ptr[v + 1]; ++q) {
-                const int32_t w = dst[q];
-                const double tw = tau[w];
-                if (!((tv < tw) || (tv == tw && v < w))) { sel = 0; break; }
-            }
-        }
-        if (sel) {
-            double cm = INFINITY;
-            int32_t lm = last[v];
-            for (int64_t q = ptr[v]; q < ptr[v + 1]; ++q) {
-                const double x = __dadd_rn(tau[dst[q]], bnd[q]);
-                if (x < cm) cm = x;
-                const int32_t lw = last[dst[q]];
-                if (lw > lm) lm = lw;
-            }
-            newt[v] = fmin(T, cm);
-            newl[v] = lm + 1;
-        }
-        flag[v] = (uint8_t)sel;
-    }
-    const int n = __syncthreads_count(sel);
-    if (threadIdx.x == 0) blockcnt[blockIdx.x] = n;
+struct PitchArgs {
+    PitchCtl* ctl;
+    int64_t nv;
+    int vpb;                    // vertices per block
+    int max_rounds;
+    double T;
+    const int64_t* ptr;
+    const int32_t* dst;
+    const double* bnd;
+    double* tau;                // [2][nv]; the launch starts from half `start`
+    int start;
+    int64_t cap;                // list entries per block
+    int32_t* lv;                // [block][cap]
+    double* lb;
+    double* lt;
+    int* cnt;                   // [round][block]
+};
+
+__device__ __forceinline__ unsigned pitch_acquire(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
 }
 
-// exclusive prefix sum of one value per thread over the block; returns the block total
-__device__ __forceinline__ int block_exclusive_scan(int x, int* excl, int* warp_tot) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int incl = x;
+__global__ void __launch_bounds__(kPitchThreads) pitch_rounds_kernel(const PitchArgs p) {
+    __shared__ int warp_cnt[kPitchThreads / 32];
+    __shared__ int s_stop;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t v0 = (int64_t)blockIdx.x * p.vpb, v1 = v0 + p.vpb < p.nv ? v0 + p.vpb : p.nv;
+    int64_t len = 0;   // entries of this block's list
+    for (int r = 0; r < p.max_rounds; ++r) {
+        const double* cur = p.tau + ((p.start + r) & 1) * p.nv;
+        double* nxt = p.tau + ((p.start + r + 1) & 1) * p.nv;
+        const int64_t before = len;
+        int done = 0;
+        for (int64_t b = v0; b < v1; b += kPitchThreads) {
+            const int64_t v = b + threadIdx.x;
+            bool sel = false;
+            double tv = 0, tn = 0;
+            if (v < v1) {
+                tv = tn = __ldcg(cur + v);
+                if (tv < p.T) {
+                    sel = true;
+                    const int64_t q1 = p.ptr[v + 1];
+                    double cm = INFINITY;
+                    for (int64_t q = p.ptr[v]; q < q1; ++q) {
+                        const int32_t w = p.dst[q];
+                        const double tw = __ldcg(cur + w);
+                        if (!((tv < tw) || (tv == tw && v < w))) { sel = false; break; }
+                        const double x = __dadd_rn(tw, p.bnd[q]);
+                        if (x < cm) cm = x;
+                    }
+                    if (sel) tn = fmin(p.T, cm);
+                }
+                __stcg(nxt + v, tn);
+                if (sel && !(tn < p.T)) ++done;
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, sel);
+            if (lane == 0) warp_cnt[warp] = __popc(m);
+            __syncthreads();
+            int off = 0, tot = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
+            for (int w = 0; w < kPitchThreads / 32; ++w) {
+                if (w < warp) off += warp_cnt[w];
+                tot += warp_cnt[w];
+            }
+            if (sel) {
+                const int64_t at = (int64_t)blockIdx.x * p.cap + len + off + __popc(m & ((1u << lane) - 1));
+                p.lv[at] = (int32_t)v;
+                p.lb[at] = tv;
+                p.lt[at] = tn;
+            }
+            len += tot;
+            __syncthreads();
+        }
+        done = __reduce_add_sync(0xffffffffu, done);
+        if (lane == 0 && done) atomicSub(&p.ctl->left, done);
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const int n = (int)(len - before);
+            p.cnt[(int64_t)r * gridDim.x + blockIdx.x] = n;
+            if (n) atomicAdd(&p.ctl->selected, n);
+            __threadfence();
+            if (atomicAdd(&p.ctl->arrived, 1u) == (unsigned)(r + 1) * gridDim.x - 1) {
+                // all blocks are here: their counts are visible, none runs on before the release
+                __threadfence();
+                const int left = *(volatile int*)&p.ctl->left, sel = *(volatile int*)&p.ctl->selected;
+                if (left == 0) p.ctl->stop = 1;
+                else if (sel == 0) p.ctl->stop = 2;
+                p.ctl->selected = 0;
+                p.ctl->rounds = r + 1;
+                __threadfence();
+                atomicExch(&p.ctl->released, (unsigned)(r + 1));
+            }
+            long long deadline = 0;
+            for (int it = 0; pitch_acquire(&p.ctl->released) < (unsigned)(r + 1); ++it) {
+                long long now;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+                if (it == 0) deadline = now + 10000000000LL;   // 10 s
+                else if (now > deadline) {
+                    atomicExch(&p.ctl->stop, 3);
+                    break;
+                }
+            }
+            s_stop = *(volatile int*)&p.ctl->stop;
+        }
+        __syncthreads();
+        if (s_stop) return;
     }
-    if (lane == 31) warp_tot[wid] = incl;
-    __syncthreads();
-    if (wid == 0) {
-        int t = lane < kPitchThreads / 32 ? warp_tot[lane] : 0;
+}
+
+// exclusive offsets of the (round, block) lists in output order, and within each block's list
+__global__ void __launch_bounds__(1024) pitch_offsets_kernel(const PitchCtl* ctl, int nblocks, const int* cnt, int64_t* out_off,
+                                                             int64_t* list_off, int64_t* round_end) {
+    __shared__ int64_t warp_sum[32];
+    const int rounds = ctl->rounds, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t n = (int64_t)rounds * nblocks;
+    int64_t carry = 0;
+    for (int64_t b = 0; b < n; b += 1024) {
+        const int64_t i = b + threadIdx.x;
+        const int64_t x = i < n ? cnt[i] : 0;
+        int64_t s = x;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, t, o);
-            if (lane >= o) t += y;
+            const int64_t y = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += y;
         }
-        warp_tot[lane] = t;   // inclusive over warps
-    }
-    __syncthreads();
-    *excl = incl - x + (wid > 0 ? warp_tot[wid - 1] : 0);
-    const int total = warp_tot[kPitchThreads / 32 - 1];
-    __syncthreads();   // warp_tot may be reused by the caller
-    return total;
-}
-
-__global__ void __launch_bounds__(kPitchThreads) pitch_scan_kernel(PitchCtl* ctl, int nblocks, const int* blockcnt,
-                                                                   int* blockoff, int64_t* layer_ptr) {
-    __shared__ int warp_tot[32];
-    if (ctl->stop) return;
-    long long carry = 0;
-    for (int b0 = 0; b0 < nblocks; b0 += kPitchThreads) {
-        const int b = b0 + (int)threadIdx.x;
-        const int x = b < nblocks ? blockcnt[b] : 0;
-        int excl;
-        const int tot = block_exclusive_scan(x, &excl, warp_tot);
-        if (b < nblocks) blockoff[b] = (int)(carry + excl);
+        if (lane == 31) warp_sum[warp] = s;
+        __syncthreads();
+        int64_t off = carry, tot = 0;
+        for (int w = 0; w < 32; ++w) {
+            if (w < warp) off += warp_sum[w];
+            tot += warp_sum[w];
+        }
+        if (i < n) {
+            out_off[i] = off + s - x;
+            if ((i + 1) % nblocks == 0) round_end[i / nblocks] = off + s;
+        }
         carry += tot;
+        __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        if (carry == 0) {
-            ctl->stop = 1;
-        } else if (ctl->count + carry > ctl->capacity || ctl->round >= ctl->layer_cap) {
-            ctl->stop = 2;
-        } else {
-            ctl->base = ctl->count;
-            ctl->count += carry;
-            ctl->cur = ctl->round;
-            layer_ptr[ctl->round + 1] = ctl->count;
-            ctl->round += 1;
+    for (int b = threadIdx.x; b < nblocks; b += 1024) {
+        int64_t s = 0;
+        for (int r = 0; r < rounds; ++r) {
+            list_off[(int64_t)r * nblocks + b] = s;
+            s += cnt[(int64_t)r * nblocks + b];
         }
     }
 }
 
-__global__ void __launch_bounds__(kPitchThreads) pitch_emit_kernel(
-    PitchCtl* ctl, int64_t nv, const uint8_t* flag, const double* newt, const int32_t* newl, const int* blockoff,
-    double* tau, int32_t* last, int32_t* out_v, double* out_tb, double* out_tt, int32_t* out_l) {
-    __shared__ int warp_tot[32];
-    if (ctl->stop) return;
-    const int64_t v = (int64_t)blockIdx.x * kPitchThreads + threadIdx.x;
-    const int sel = v < nv ? (int)flag[v] : 0;
-    int rank;
-    block_exclusive_scan(sel, &rank, warp_tot);
-    if (sel) {
-        const long long pos = ctl->base + blockoff[blockIdx.x] + rank;
-        const int32_t l = newl[v];
-        out_v[pos] = (int32_t)v;
-        out_tb[pos] = tau[v];
-        out_tt[pos] = newt[v];
-        out_l[pos] = l;
-        if (l != ctl->cur) atomicExch(&ctl->err, 1);
-        tau[v] = newt[v];
-        last[v] = l;
-    }
-}
-
-__global__ void pitch_init_kernel(int64_t nv, double* tau, int32_t* last) {
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += (int64_t)gridDim.x * blockDim.x) {
-        tau[v] = 0.0;
-        last[v] = -1;
+__global__ void __launch_bounds__(kPitchThreads) pitch_order_kernel(const PitchCtl* ctl, const int* cnt, const int64_t* out_off,
+                                                                    const int64_t* list_off, int64_t cap, const int32_t* lv,
+                                                                    const double* lb, const double* lt, int32_t* ov, double* ob,
+                                                                    double* ot) {
+    const int rounds = ctl->rounds, nb = gridDim.x, lane = threadIdx.x & 31;
+    for (int r = threadIdx.x >> 5; r < rounds; r += kPitchThreads / 32) {
+        const int64_t k = (int64_t)r * nb + blockIdx.x, from = blockIdx.x * cap + list_off[k], to = out_off[k];
+        for (int i = lane; i < cnt[k]; i += 32) {
+            ov[to + i] = lv[from + i];
+            ob[to + i] = lb[from + i];
+            ot[to + i] = lt[from + i];
+        }
     }
 }
 
@@ -176,8 +219,7 @@ namespace {
 struct PitchBuffers {
     std::vector<void*> owned;
     ~PitchBuffers() {
-        for (void* p : owned)
-            if (p) cudaFree(p);
+        for (void* p : owned) cudaFree(p);
     }
     template <typename T>
     cudaError_t alloc(T** p, size_t n) {
@@ -186,24 +228,6 @@ struct PitchBuffers {
         if (e == cudaSuccess) owned.push_back(*p);
         return e;
     }
-    // replace *p (n_old valid entries) by a buffer of n_new entries
-    template <typename T>
-    cudaError_t grow(T** p, size_t n_old, size_t n_new, cudaStream_t st) {
-        T* q = nullptr;
-        cudaError_t e = alloc(&q, n_new);
-        if (e != cudaSuccess) return e;
-        if (n_old) e = cudaMemcpyAsync(q, *p, n_old * sizeof(T), cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return e;
-        e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return e;
-        for (void*& o : owned)
-            if (o == (void*)*p) {
-                cudaFree(o);
-                o = nullptr;
-            }
-        *p = q;
-        return cudaSuccess;
-    }
 };
 
 }  // namespace
@@ -211,104 +235,96 @@ struct PitchBuffers {
 int device_pitch(const Mesh& m, const PitchGraph& g, double T, Tents& out, void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
     const int64_t nv = m.nv;
-    const int nblocks = (int)((nv + kPitchThreads - 1) / kPitchThreads);
+    // blocks: one vertex per thread as long as all blocks are resident together
+    int dev = 0, nsm = 0, per_sm = 0;
+    PITCH_TRY(cudaGetDevice(&dev));
+    PITCH_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    PITCH_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pitch_rounds_kernel, kPitchThreads, 0));
+    const int64_t resident = (int64_t)std::max(1, per_sm) * nsm;
+    int64_t vpt = 1;
+    while ((nv + vpt * kPitchThreads - 1) / (vpt * kPitchThreads) > resident) ++vpt;
+    const int nblocks = (int)((nv + vpt * kPitchThreads - 1) / (vpt * kPitchThreads));
+    PitchArgs p{};
+    p.nv = nv;
+    p.vpb = (int)(vpt * kPitchThreads);
+    p.T = T;
+    // a list holds every round's tents of a block: at most every vertex once a round; bounded memory
+    p.max_rounds = (int)std::max<int64_t>(8, std::min<int64_t>(kPitchChunk, ((int64_t)1 << 25) / nv));
+    p.cap = (int64_t)p.vpb * p.max_rounds;
     PitchBuffers B;
-    int64_t* d_ptr;
-    int32_t* d_dst;
-    double* d_bnd;
-    double *d_tau, *d_newt;
-    int32_t *d_last, *d_newl;
-    uint8_t* d_flag;
-    int *d_bcnt, *d_boff;
-    PitchCtl* d_ctl;
+    int64_t *d_ptr, *d_out_off, *d_list_off, *d_round_end;
+    int32_t *d_dst, *o_v;
+    double *d_bnd, *o_b, *o_t;
+    const size_t list = (size_t)nblocks * p.cap, cells = (size_t)p.max_rounds * nblocks;
+    PITCH_TRY(B.alloc(&p.ctl, 1));
     PITCH_TRY(B.alloc(&d_ptr, g.ptr.size()));
     PITCH_TRY(B.alloc(&d_dst, g.dst.size()));
     PITCH_TRY(B.alloc(&d_bnd, g.bnd.size()));
-    PITCH_TRY(B.alloc(&d_tau, nv));
-    PITCH_TRY(B.alloc(&d_newt, nv));
-    PITCH_TRY(B.alloc(&d_last, nv));
-    PITCH_TRY(B.alloc(&d_newl, nv));
-    PITCH_TRY(B.alloc(&d_flag, nv));
-    PITCH_TRY(B.alloc(&d_bcnt, nblocks));
-    PITCH_TRY(B.alloc(&d_boff, nblocks));
-    PITCH_TRY(B.alloc(&d_ctl, 1));
+    PITCH_TRY(B.alloc(&p.tau, 2 * nv));
+    PITCH_TRY(B.alloc(&p.lv, list));
+    PITCH_TRY(B.alloc(&p.lb, list));
+    PITCH_TRY(B.alloc(&p.lt, list));
+    PITCH_TRY(B.alloc(&p.cnt, cells));
+    PITCH_TRY(B.alloc(&d_out_off, cells));
+    PITCH_TRY(B.alloc(&d_list_off, cells));
+    PITCH_TRY(B.alloc(&d_round_end, p.max_rounds));
+    PITCH_TRY(B.alloc(&o_v, list));
+    PITCH_TRY(B.alloc(&o_b, list));
+    PITCH_TRY(B.alloc(&o_t, list));
+    p.ptr = d_ptr;
+    p.dst = d_dst;
+    p.bnd = d_bnd;
     PITCH_TRY(cudaMemcpyAsync(d_ptr, g.ptr.data(), g.ptr.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st));
     if (!g.dst.empty()) {
         PITCH_TRY(cudaMemcpyAsync(d_dst, g.dst.data(), g.dst.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
         PITCH_TRY(cudaMemcpyAsync(d_bnd, g.bnd.data(), g.bnd.size() * sizeof(double), cudaMemcpyHostToDevice, st));
     }
-    pitch_init_kernel<<<(int)std::min<int64_t>(nblocks, 1024), kPitchThreads, 0, st>>>(nv, d_tau, d_last);
-    PITCH_TRY(cudaGetLastError());
-
-    // output arrays, grown when a round does not fit (the round is then run again)
-    size_t cap = (size_t)std::max<int64_t>(nv * 16, 1 << 16);
-    int layer_cap = 4096;
-    int32_t *o_v, *o_l;
-    double *o_tb, *o_tt;
-    int64_t* d_lptr;
-    PITCH_TRY(B.alloc(&o_v, cap));
-    PITCH_TRY(B.alloc(&o_l, cap));
-    PITCH_TRY(B.alloc(&o_tb, cap));
-    PITCH_TRY(B.alloc(&o_tt, cap));
-    PITCH_TRY(B.alloc(&d_lptr, (size_t)layer_cap + 1));
-    PITCH_TRY(cudaMemsetAsync(d_lptr, 0, sizeof(int64_t), st));
+    PITCH_TRY(cudaMemsetAsync(p.tau, 0, 2 * nv * sizeof(double), st));
+    out.layer_ptr.assign(1, 0);
     PitchCtl h{};
-    h.capacity = (long long)cap;
-    h.layer_cap = layer_cap;
-    PITCH_TRY(cudaMemcpyAsync(d_ctl, &h, sizeof(h), cudaMemcpyHostToDevice, st));
+    h.left = (int)nv;
+    std::vector<int64_t> ends(p.max_rounds);
+    long long rounds = 0;
     while (true) {
-        for (int r = 0; r < kPitchRoundsPerSync; ++r) {
-            pitch_select_kernel<<<nblocks, kPitchThreads, 0, st>>>(d_ctl, nv, T, d_ptr, d_dst, d_bnd, d_tau, d_last,
-                                                                   d_flag, d_newt, d_newl, d_bcnt);
-            pitch_scan_kernel<<<1, kPitchThreads, 0, st>>>(d_ctl, nblocks, d_bcnt, d_boff, d_lptr);
-            pitch_emit_kernel<<<nblocks, kPitchThreads, 0, st>>>(d_ctl, nv, d_flag, d_newt, d_newl, d_boff, d_tau,
-                                                                 d_last, o_v, o_tb, o_tt, o_l);
-        }
+        h.arrived = h.released = 0;
+        h.rounds = 0;
+        PITCH_TRY(cudaMemcpyAsync(p.ctl, &h, sizeof(h), cudaMemcpyHostToDevice, st));
+        void* args[] = {&p};
+        PITCH_TRY(cudaLaunchCooperativeKernel((const void*)pitch_rounds_kernel, dim3(nblocks), dim3(kPitchThreads), args, 0, st));
+        pitch_offsets_kernel<<<1, 1024, 0, st>>>(p.ctl, nblocks, p.cnt, d_out_off, d_list_off, d_round_end);
+        pitch_order_kernel<<<nblocks, kPitchThreads, 0, st>>>(p.ctl, p.cnt, d_out_off, d_list_off, p.cap, p.lv, p.lb, p.lt, o_v,
+                                                              o_b, o_t);
         PITCH_TRY(cudaGetLastError());
-        PITCH_TRY(cudaMemcpyAsync(&h, d_ctl, sizeof(h), cudaMemcpyDeviceToHost, st));
+        PITCH_TRY(cudaMemcpyAsync(&h, p.ctl, sizeof(h), cudaMemcpyDeviceToHost, st));
+        PITCH_TRY(cudaMemcpyAsync(ends.data(), d_round_end, p.max_rounds * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
         PITCH_TRY(cudaStreamSynchronize(st));
-        if (h.err) return set_error(MTP_ECUDA, "device pitcher: a tent's layer differs from its round (internal error)");
+        if (h.stop == 3) return set_error(MTP_ETIMEOUT, "device pitcher: a wait between rounds exceeded the limit");
+        // a round that selected nothing adds no layer
+        const int nr = h.stop == 2 ? h.rounds - 1 : h.rounds;
+        const int64_t n0 = (int64_t)out.vertex.size(), n = nr > 0 ? ends[nr - 1] : 0;
+        out.vertex.resize(n0 + n);
+        out.layer.resize(n0 + n);
+        out.t_bot.resize(n0 + n);
+        out.t_top.resize(n0 + n);
+        if (n) {
+            PITCH_TRY(cudaMemcpyAsync(out.vertex.data() + n0, o_v, n * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+            PITCH_TRY(cudaMemcpyAsync(out.t_bot.data() + n0, o_b, n * sizeof(double), cudaMemcpyDeviceToHost, st));
+            PITCH_TRY(cudaMemcpyAsync(out.t_top.data() + n0, o_t, n * sizeof(double), cudaMemcpyDeviceToHost, st));
+        }
+        for (int r = 0; r < nr; ++r) {
+            const int64_t from = r ? ends[r - 1] : 0;
+            std::fill(out.layer.begin() + n0 + from, out.layer.begin() + n0 + ends[r], (int32_t)(rounds + r));
+            out.layer_ptr.push_back(n0 + ends[r]);
+        }
+        PITCH_TRY(cudaStreamSynchronize(st));
+        rounds += nr;
+        p.start = (p.start + h.rounds) & 1;
         if (h.stop == 1) break;
-        if (h.round > kPitchMaxRounds)
+        if (h.stop == 2) return set_error(MTP_ECAUSAL, "pitching stalled before reaching T");
+        if (rounds > kPitchMaxRounds)
             return set_error(MTP_ECAUSAL, "device pitcher: no end after " + std::to_string(kPitchMaxRounds) +
                                               " rounds (edge bounds below the resolution of tau?)");
-        if (h.stop == 2) {   // the pending round did not fit: grow and run it again
-            if (h.round >= h.layer_cap) {
-                const int nc = h.layer_cap * 2;
-                PITCH_TRY(B.grow(&d_lptr, (size_t)h.layer_cap + 1, (size_t)nc + 1, st));
-                h.layer_cap = nc;
-            } else {
-                const size_t nc = std::max<size_t>(cap * 2, (size_t)h.count + (size_t)nv);
-                PITCH_TRY(B.grow(&o_v, (size_t)h.count, nc, st));
-                PITCH_TRY(B.grow(&o_l, (size_t)h.count, nc, st));
-                PITCH_TRY(B.grow(&o_tb, (size_t)h.count, nc, st));
-                PITCH_TRY(B.grow(&o_tt, (size_t)h.count, nc, st));
-                cap = nc;
-                h.capacity = (long long)cap;
-            }
-            h.stop = 0;
-            PITCH_TRY(cudaMemcpyAsync(d_ctl, &h, sizeof(h), cudaMemcpyHostToDevice, st));
-        }
     }
-    const size_t n = (size_t)h.count;
-    const int64_t nl = h.round;
-    out.vertex.resize(n);
-    out.layer.resize(n);
-    out.t_bot.resize(n);
-    out.t_top.resize(n);
-    out.layer_ptr.resize(nl + 1);
-    std::vector<double> tau(nv);
-    if (n) {
-        PITCH_TRY(cudaMemcpyAsync(out.vertex.data(), o_v, n * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        PITCH_TRY(cudaMemcpyAsync(out.layer.data(), o_l, n * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        PITCH_TRY(cudaMemcpyAsync(out.t_bot.data(), o_tb, n * sizeof(double), cudaMemcpyDeviceToHost, st));
-        PITCH_TRY(cudaMemcpyAsync(out.t_top.data(), o_tt, n * sizeof(double), cudaMemcpyDeviceToHost, st));
-    }
-    PITCH_TRY(cudaMemcpyAsync(out.layer_ptr.data(), d_lptr, (nl + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    PITCH_TRY(cudaMemcpyAsync(tau.data(), d_tau, nv * sizeof(double), cudaMemcpyDeviceToHost, st));
-    PITCH_TRY(cudaStreamSynchronize(st));
-    for (int64_t v = 0; v < nv; ++v)
-        if (tau[v] != T) return set_error(MTP_ECAUSAL, "pitching stalled before reaching T");
     return MTP_OK;
 }
 
