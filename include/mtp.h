@@ -164,17 +164,17 @@ int mtp_state_to_lattice(mtp_mesh_t mesh, const void* state_dev, double* vals_de
 int mtp_evolve(mtp_tents_t tents, void* state_dev, double T, void* stream);
 
 /* Evolve launch configuration of this tents handle: 0 (default) the persistent DAG walk with as
- * many CTAs per SM as fit, 1 the DAG walk with one CTA per SM, 2 one launch per layer (CUDA
+ * many CTAs per SM as fit and as the average layer fills, 1 the DAG walk with one CTA per SM, 2 one launch per layer (CUDA
  * graph).  MTP_FLAG_LAYER_LAUNCHES on the mesh forces 2. */
 int mtp_tents_set_launch(mtp_tents_t tents, int launch);
 
-/* Kernel shape variant of this tents handle (MTP_FP32 SAT meshes): 0 (default) each stage item
- * of the tent kernel covers a pair of patch elements with the same local index of the tent
- * vertex, which share every reference-table read; 1 each item covers one element: twice the
- * items at half the work each, so a tent finishes sooner when the layers hold fewer tents than
- * the GPU has CTA slots (e.g. small meshes), at a lower throughput when they hold more;
- * 2 each item covers one element and one basis function (or facet mode), with 512 threads per
- * CTA in 3D: the shortest tents for such latency-bound layers.  3 and 4 (3D, p = 2..4, patches
+/* Kernel shape variant of this tents handle (MTP_FP32 SAT meshes).  In 2D, and in 3D up to p = 4,
+ * variants 0, 1 and 2 all select the apex tent kernel, which is the fastest for every layer width.
+ * For 3D p = 5: 0 (default) each stage item of the tent kernel covers a pair of patch elements with
+ * the same local index of the tent vertex, which share every reference-table read; 1 each item
+ * covers one element: twice the items at half the work each, so a tent finishes sooner when the
+ * layers hold fewer tents than the GPU has CTA slots; 2 each item covers one element and one basis
+ * function (or facet mode), with 512 threads per CTA.  3 and 4 (3D, p = 2..4, patches
  * of at most 42 tetrahedra): the item shapes of 1 and 2 on 512 threads, with the volume term of
  * the operator (Sec. 3, the element integrals of the DG semi-discretisation) computed on the
  * tcgen05 tensor cores as TF32 MMAs with a three-term hi + lo operand split and FP32
@@ -222,7 +222,8 @@ int mtp_batch_evolve(mtp_batch_t batch, void* const* states_dev, void* stream);
  * right-hand sides) = the derivatives of J through the tent maps' dependence on eps and mu
  * (the mass operator g(u) - f(u) grad(phi) and the facet impedances).  Dependence of the
  * initial state or of J on eps, mu is the caller's to add.  The forward pass keeps the state
- * before every checkpoint_every-th layer (0: about sqrt(n_layers)); each segment is
+ * before every checkpoint_every-th layer (0: all layers form one segment when their patch tape
+ * takes at most 4 GB, about sqrt(n_layers) otherwise); each segment is
  * recomputed from its checkpoint and reversed layer by layer, one CTA per tent, replaying
  * the tent's SAT stages into a device tape.  Device work buffers are owned by the tents
  * handle.  Completion and errors as for mtp_evolve; MTP_EUNSUPPORTED if the adjoint kernel's

@@ -14,6 +14,8 @@
 // Material gradients: each solve contributes -nu^T (dM/dp) U (dM/deps = E block, dM/dmu = H
 // block); A depends on eps, mu through Z = sqrt(mu/eps) in the fluxes: dJ/dZ from forward-mode
 // dual numbers through the same flux routine, then dZ/deps = -Z/(2 eps), dZ/dmu = Z/(2 mu).
+//
+// This general form serves 2D and 3D degrees beyond the apex kernels'; mtp_apex_adjoint.cuh is the other.
 #pragma once
 
 #include "mtp_kernels.cuh"

@@ -161,10 +161,25 @@ struct ApexTent {
     // C lies on the first, D on the second, B on both; C and D also lie on the facet opposite B.
     template <int WT>
     __device__ __forceinline__ void phase_traces() {
+        Real u[NB];
+        apex_load<NB>(ucol(3 * f + (WT < 0 ? w : WT)), lane, u);
+        traces_of<WT, false>(u, sTr());
+    }
+    // LAM: the traces times lambda_V (used by the adjoint)
+    template <int WT, bool LAM>
+    __device__ __forceinline__ void traces_of(const Real* u, Real* buf) {
         constexpr int NS = Op::NS;
         const int W = WT < 0 ? w : WT;
-        Real u[NB];
-        apex_load<NB>(ucol(3 * f + W), lane, u);
+        auto put = [&](int fi, int fs, const Real* t) {
+            Real* to = buf + (fi * 4 + fs) * Sh::GF * COL;
+            if constexpr (LAM) {
+                Real g[NFB];
+                Op::lam(t, g);
+                apex_store<NFB>(to, lane, g);
+            } else {
+                apex_store<NFB>(to, lane, t);
+            }
+        };
         {
             Real e[NS], o[NS];
             Op::pair_even(u, e);
@@ -174,7 +189,7 @@ struct ApexTent {
 #pragma unroll
                 for (int q = 0; q < NS; ++q) s[q] = WT < 0 ? e[q] + (fi ? Real(1) : Real(-1)) * o[q] : fi ? e[q] + o[q] : e[q] - o[q];
                 Op::pair_trace(s, t);
-                apex_store<NFB>(tr(fi, 2 * f + (W == 2 ? 1 : 0)), lane, t);
+                put(fi, 2 * f + (W == 2 ? 1 : 0), t);
             };
             if constexpr (WT >= 0) {
                 if (W != 0) facet(0);
@@ -192,7 +207,7 @@ struct ApexTent {
         if (W != 2) {
             Real t[NFB];
             Op::trace2(u, t);
-            apex_store<NFB>(tr(2, 2 * f + W), lane, t);
+            put(2, 2 * f + W, t);
         }
     }
 
@@ -374,8 +389,9 @@ struct ApexTent {
         return K;
     }
 
-    // U = K r for the vectors of coefficients of this warp
-    __device__ __forceinline__ void phase_solve(const Mass& K) {
+    // U = K r for the vectors of coefficients of this warp (TAPE: also into a tape slot)
+    template <bool TAPE = false>
+    __device__ __forceinline__ void phase_solve(const Mass& K, Real* tape = nullptr) {
         using VT = typename Vec<Real>::T;
         constexpr int VW = Sh::VW;
 #pragma unroll 1
@@ -400,7 +416,10 @@ struct ApexTent {
                 r[5][v] = K.m[2] * h[0] + K.m[4] * h[1] + K.m[5] * h[2] + (K.c[0] * e1 - K.c[1] * e0);
             }
 #pragma unroll
-            for (int c = 0; c < 6; ++c) *(VT*)(ucol(c) + (g * 32 + lane) * VW) = apex_pack(r[c]);
+            for (int c = 0; c < 6; ++c) {
+                *(VT*)(ucol(c) + (g * 32 + lane) * VW) = apex_pack(r[c]);
+                if constexpr (TAPE) *(VT*)(tape + (c * Sh::GB + g) * COL + lane * VW) = apex_pack(r[c]);
+            }
         }
     }
 
@@ -508,36 +527,59 @@ struct ApexTent {
         return (Real)fmax(head()->tt - head()->tb, sizeof(Real) == 4 ? 1e-30 : 1e-200);
     }
 
+    // patch coefficients (library layout) into the staging buffer
+    template <bool CG>
+    __device__ __forceinline__ void stage_patch(const Real* state) {
+        constexpr int NC = 6 * NB, STEP = 8;   // loads in flight
+        const int ns = head()->ns;
+        for (int i0 = threadIdx.x; i0 < ns * NC; i0 += STEP * Sh::NT) {
+            Real v[STEP];
+#pragma unroll
+            for (int q = 0; q < STEP; ++q) {
+                const int idx = i0 + q * Sh::NT, e = idx / NC, r = idx - e * NC;
+                if (idx < ns * NC) {
+                    const Real* sp = state + (int64_t)sElem()[e] * NC + r;
+                    v[q] = CG ? __ldcg(sp) : *sp;
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < STEP; ++q) {
+                const int idx = i0 + q * Sh::NT, e = idx / NC, r = idx - e * NC;
+                if (idx < ns * NC) sTr()[e * Sh::SP + r] = v[q];
+            }
+        }
+    }
+    // own component of the staged patch along the record's vectors at `vec`, in the apex basis
+    __device__ __forceinline__ void component_in(const KArgs& a, int vec, Real sc, Real* z) {
+        const int ns = head()->ns, k = lane < ns ? lane : ns - 1, j = *(const int8_t*)(sInfo() + 3 * k);
+        const Real* rec = (const Real*)head()->ent + k * kApexRec + vec + 3 * w;
+        const Real g0 = __ldg(rec), g1 = __ldg(rec + 1), g2 = __ldg(rec + 2);
+        const Real* st = sTr() + k * Sh::SP + f * 3 * NB;
+        Real y[NB];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) y[b] = g0 * st[b] + g1 * st[NB + b] + g2 * st[2 * NB + b];
+        rotate<true>((const Real*)a.Rt + (size_t)j * apex_rot_offset(P + 1), y, z);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) z[b] *= sc;
+    }
+
     // The tent for one right-hand side: read the patch, evolve bottom to top, write the patch.
     // CG: other CTAs of the same launch write the state and the front (bypass L1).
     template <bool CG>
     __device__ void run(const KArgs& a, Real* state) {
-        constexpr int NC = 6 * NB;
+        begin<CG>(a, state);
+        Real dl[NB];
+        stages<false>(a, dl, nullptr);
+        finish<CG>(a, state, dl, kApexEdge, (f ? Real(1) : Real(-1)) * height() * cst(18, lane));
+    }
+
+    // read the patch and the front; y0 into its buffer and r
+    template <bool CG>
+    __device__ __forceinline__ void begin(const KArgs& a, const Real* state) {
         __syncthreads();
         const double tb = head()->tb, dtd = head()->tt - tb;
-        const int ns = head()->ns, k = lane < ns ? lane : ns - 1;
-        const Real* ent = (const Real*)head()->ent;
-        const int8_t* inf = (const int8_t*)(sInfo() + 3 * k);
-        const int j = inf[0];
-        {
-            constexpr int STEP = 8;   // loads in flight
-            for (int i0 = threadIdx.x; i0 < ns * NC; i0 += STEP * Sh::NT) {
-                Real v[STEP];
-#pragma unroll
-                for (int q = 0; q < STEP; ++q) {
-                    const int idx = i0 + q * Sh::NT, e = idx / NC, r = idx - e * NC;
-                    if (idx < ns * NC) {
-                        const Real* sp = state + (int64_t)sElem()[e] * NC + r;
-                        v[q] = CG ? __ldcg(sp) : *sp;
-                    }
-                }
-#pragma unroll
-                for (int q = 0; q < STEP; ++q) {
-                    const int idx = i0 + q * Sh::NT, e = idx / NC, r = idx - e * NC;
-                    if (idx < ns * NC) sTr()[e * Sh::SP + r] = v[q];
-                }
-            }
-        }
+        const int ns = head()->ns, k = lane < ns ? lane : ns - 1, j = *(const int8_t*)(sInfo() + 3 * k);
+        stage_patch<CG>(state);
         double* chk = (double*)((unsigned char*)sTr() + Sh::CHECK);
         const int32_t* verts = a.elems + (int64_t)sElem()[lane] * 4;
         if (f == 0) {   // covariant components of grad phi at the tent bottom
@@ -564,32 +606,25 @@ struct ApexTent {
             if (!(chk[lane] + chk[64 + lane] + chk[128 + lane] < em) || !(chk[32 + lane] + chk[96 + lane] + chk[160 + lane] < em))
                 atomicCAS(a.err, 0, 1);
         }
+        Real z[NB];
+        component_in(a, kApexDual, (f ? Real(1) : Real(-1)) * cst(17, k) / height(), z);
+        apex_store<NB>(sY0() + (3 * f + w) * Sh::GB * COL, lane, z);
+        apex_store<NB>(rcol(3 * f + w), lane, z);
+        __syncthreads();
+    }
+
+    // all m q stages; dl receives the increment.  TAPE: U_{i,n} of every stage to slot i q + n.
+    template <bool TAPE>
+    __device__ __forceinline__ void stages(const KArgs& a, Real* dl, Real* tape) {
+        constexpr int SLOT = 6 * Sh::GB * COL;
         const int nown = head()->nown;
         const float inv_nown = 1.0f / (float)nown;
-        const Real dt = height(), sgn = f ? Real(1) : Real(-1);
-        const Real* Rt = (const Real*)a.Rt + (size_t)j * apex_rot_offset(P + 1);
-        Real dl[NB];
-        {
-            Real y[NB], z[NB];
-            const Real* rec = ent + k * kApexRec + kApexDual + 3 * w;
-            const Real g0 = __ldg(rec), g1 = __ldg(rec + 1), g2 = __ldg(rec + 2);
-            const Real* st = sTr() + k * Sh::SP + f * 3 * NB;
+        const Real dt = height();
 #pragma unroll
-            for (int b = 0; b < NB; ++b) y[b] = g0 * st[b] + g1 * st[NB + b] + g2 * st[2 * NB + b];
-            rotate<true>(Rt, y, z);
-            const Real sc = sgn * cst(17, k) / dt;
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
-                z[b] *= sc;
-                dl[b] = Real(0);
-            }
-            apex_store<NB>(sY0() + (3 * f + w) * Sh::GB * COL, lane, z);
-            apex_store<NB>(rcol(3 * f + w), lane, z);
-        }
-        __syncthreads();
+        for (int b = 0; b < NB; ++b) dl[b] = Real(0);
         for (int i = 0; i < a.m; ++i) {
             const Mass K = mass_at(dt, sSub()[i]);
-            phase_solve(K);
+            phase_solve<TAPE>(K, tape + (size_t)i * a.q * SLOT);
             __syncthreads();
             for (int n = 1; n <= a.q; ++n) {
                 by_component([&](auto W) { phase_traces<decltype(W)::value>(); });
@@ -617,18 +652,16 @@ struct ApexTent {
                 apex_store<NB>(rcol(3 * f + w), lane, acc);
                 __syncthreads();
                 if (!last) {
-                    phase_solve(K);
+                    phase_solve<TAPE>(K, tape + (size_t)(i * a.q + n) * SLOT);
                     __syncthreads();
                 }
             }
         }
-        // back to the library basis; the staging buffer shares the trace and U buffers (all read)
-        finish<CG>(a, state, dl);
     }
 
-    // add the increment to the state
-    template <bool CG>
-    __device__ __forceinline__ void finish(const KArgs& a, Real* state, const Real* dl) {
+    // state += the own components dl (apex basis) times sc along the record's vectors at `vec`
+    template <bool CG, bool CHECK = true>
+    __device__ __forceinline__ void finish(const KArgs& a, Real* state, const Real* dl, int vec, Real sc) {
         constexpr int NC = 6 * NB;
         const int ns = head()->ns, k = lane < ns ? lane : ns - 1;
         const Real* ent = (const Real*)head()->ent;
@@ -636,8 +669,7 @@ struct ApexTent {
             const int j = *(const int8_t*)(sInfo() + 3 * k);
             Real z[NB];
             rotate<false>((const Real*)a.Rt + (size_t)j * apex_rot_offset(P + 1), dl, z);
-            const Real sc = (f ? Real(1) : Real(-1)) * height() * cst(18, k);
-            __syncthreads();
+            __syncthreads();   // the staging buffer shares the trace and U buffers (all read)
             Real* st = sTr() + k * Sh::SP + (3 * f + w) * NB;
             if (lane < ns)
 #pragma unroll
@@ -648,10 +680,10 @@ struct ApexTent {
         for (int idx = threadIdx.x; idx < ns * NC; idx += Sh::NT) {
             const int e = idx / NC, r = idx - e * NC, c = r / NB, b = r - c * NB, fl = c / 3, x = c - 3 * fl;
             const Real* st = sTr() + e * Sh::SP + fl * 3 * NB + b;
-            const Real* t = ent + e * kApexRec + kApexEdge + x;
+            const Real* t = ent + e * kApexRec + vec + x;
             Real* sp = state + (int64_t)sElem()[e] * NC + r;
             const Real v = (CG ? __ldcg(sp) : *sp) + (__ldg(t) * st[0] + __ldg(t + 3) * st[NB] + __ldg(t + 6) * st[2 * NB]);
-            if (!isfinite(v)) bad = true;
+            if (CHECK && !isfinite(v)) bad = true;
             *sp = v;
         }
         if (bad) atomicCAS(a.err, 0, 2);

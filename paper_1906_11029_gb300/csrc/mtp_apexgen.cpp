@@ -176,6 +176,11 @@ void emit_degree(FILE* f, int p) {
     emit(f, "vol_ab", transpose(along(0, 1, -1)), true);     // along B - A
     emit(f, "vol_mb", transpose(along(-0.5, 1, 0)), true);   // along B - (C + D) / 2
     emit(f, "vol_cd", transpose(along(1, 0, 0)), true);      // along D - C
+    // the same for the adjoint: rows c, and lambda_V transposed
+    emit(f, "volt_ab", along(0, 1, -1), false);
+    emit(f, "volt_mb", along(-0.5, 1, 0), true);
+    emit(f, "volt_cd", along(1, 0, 0), true);
+    emit(f, "mass_t", transpose(M), true);
     std::fprintf(f, "};\n\n");
 }
 

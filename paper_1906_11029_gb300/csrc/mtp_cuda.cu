@@ -345,7 +345,8 @@ static int apex2_upload_real(const Mesh& m, DeviceMesh& d) {
     return MTP_OK;
 }
 
-// the apex tent kernels run the plain SAT modes in 2D, and in 3D up to kApexMaxDegree
+// the apex tent kernels run the plain SAT modes in 2D, and these and the adjoint in 3D up to
+// kApexMaxDegree
 static int apex_upload(const Mesh& m, DeviceMesh& d) {
     if (m.dim == 2) {
         if (m.precision == MTP_FP64) return apex2_upload_real<double>(m, d);
@@ -353,7 +354,8 @@ static int apex_upload(const Mesh& m, DeviceMesh& d) {
     }
     if (m.p > kApexMaxDegree) return MTP_OK;
     if (m.precision == MTP_FP64) return apex_upload_real<double>(m, d);
-    return m.precision == MTP_FP32 ? apex_upload_real<float>(m, d) : MTP_OK;
+    // the tensor-core modes' adjoint runs in FP32
+    return m.precision == MTP_FP32_SPLIT ? MTP_OK : apex_upload_real<float>(m, d);
 }
 
 int device_mesh_upload(Mesh& m) {
@@ -791,9 +793,6 @@ int device_adjoint(Tents& t, const void* state0, const void* lamT, void* lam0, d
     CUDA_TRY(pa_);
     CUDA_TRY(pf_);
     const int64_t nl = (int64_t)t.layer_ptr.size() - 1;
-    if (K <= 0) K = std::max<int64_t>(1, (int64_t)std::ceil(std::sqrt((double)nl)));
-    K = std::min(K, nl);
-    const int64_t nck = (nl + K - 1) / K;
     const size_t sbytes = (size_t)m.n_rhs * m.ne * m.nf * m.nb * real_size(m);
     int64_t max_tents = 0;
     for (int64_t l = 0; l < nl; ++l) max_tents = std::max(max_tents, t.layer_ptr[l + 1] - t.layer_ptr[l]);
@@ -802,6 +801,16 @@ int device_adjoint(Tents& t, const void* state0, const void* lamT, void* lam0, d
     for (size_t i = 0; i < t.vertex.size(); ++i)
         off[i + 1] = off[i] + (m.patch_ptr[t.vertex[i] + 1] - m.patch_ptr[t.vertex[i]]);
     if (!d.tent_off) MTP_TRY(upload(&d.tent_off, off.data(), off.size()));
+    if (K <= 0) {
+        // One segment when the patch tape of the whole evolve stays within kAdjointTape: nothing is
+        // computed twice (adjoint workload 8^3, p = 2: 98 MB).  About sqrt(layers) otherwise, which
+        // balances checkpoints and tape at the price of a second forward pass.
+        constexpr size_t kAdjointTape = (size_t)4 << 30;
+        const size_t whole = (size_t)off.back() * m.n_rhs * m.nf * m.nb * real_size(m);
+        K = whole <= kAdjointTape ? nl : std::max<int64_t>(1, (int64_t)std::ceil(std::sqrt((double)nl)));
+    }
+    K = std::min(K, nl);
+    const int64_t nck = (nl + K - 1) / K;
     int64_t seg_entries = 0;
     for (int64_t c = 0; c < nck; ++c) {
         const int64_t l0 = c * K, l1 = std::min((c + 1) * K, nl);
@@ -834,8 +843,9 @@ int device_adjoint(Tents& t, const void* state0, const void* lamT, void* lam0, d
     KArgs fa;
     for (int64_t c = 0; c < nck; ++c) {
         CUDA_TRY(cudaMemcpyAsync(ckpt(c), work, sbytes, cudaMemcpyDeviceToDevice, st));
+        if (c + 1 == nck) break;   // the last segment's layers run when it is reversed
         fill_args(t, work, fa);
-        MTP_TRY(enqueue_layers(t, fa, c * K, std::min((c + 1) * K, nl), st));
+        MTP_TRY(enqueue_layers(t, fa, c * K, (c + 1) * K, st));
     }
     // reverse sweep
     CUDA_TRY(cudaMemcpyAsync(lam0, lamT, sbytes, cudaMemcpyDeviceToDevice, st));

@@ -163,3 +163,42 @@ def test_vertex_without_elements(dim):
             tents.evolve(st)
             outs.append(st)
     assert all(torch.equal(outs[0], o) for o in outs[1:])
+
+
+@pytest.mark.parametrize("name,p", [("cube2", 1), ("cube2", 2), ("ball32", 2), ("one_tet", 2), ("cube2", 3)])
+def test_apex_adjoint_matches_directional_differences(name, p):
+    """Gradients w.r.t. the initial state, eps and mu along one direction each against central differences of
+    FP64 evolves (h = 1e-6: about 1e-9 of rounding and h^2 of truncation; FP32 adds its own 1e-5)."""
+    v, e, eps, mu = _problem(name)
+    T = 0.05
+    rng = np.random.default_rng(p)
+    ws = np.ones(len(e))
+    ref = mtp.Mesh(3, v, e, eps, mu, p=p)
+    Y0 = torch.tensor(rng.standard_normal(ref.state_shape), device=DEV)
+    dY, de, dm = torch.tensor(rng.standard_normal(ref.state_shape), device=DEV), rng.standard_normal(len(e)), rng.standard_normal(len(e))
+
+    def J(h, which):
+        m = mtp.Mesh(3, v, e, eps + (h * de if which == 1 else 0), mu + (h * dm if which == 2 else 0), p=p)
+        Y = Y0 + h * dY if which == 0 else Y0.clone()
+        m.pitch(T, 0.5, wavespeed=ws).evolve(Y)
+        return 0.5 * Y.square().sum().item()
+
+    want = [(J(1e-6, k) - J(-1e-6, k)) / 2e-6 for k in range(3)]
+    scale = Y0.square().sum().item()
+    for prec, tol in ((mtp.MTP_FP64, 1e-8), (mtp.MTP_FP32, 1e-5)):
+        if prec == mtp.MTP_FP64 and p > 2:
+            continue    # the differences above cover the forward; cube2's FP64 gradients run at p = 1, 2
+        m = mtp.Mesh(3, v, e, eps, mu, p=p, precision=prec)
+        t = m.pitch(T, 0.5, wavespeed=ws)
+        for every in (0, 3):
+            Y = Y0.to(m.torch_dtype()).requires_grad_(True)
+            pe, pm = (torch.tensor(x, device=DEV, requires_grad=True) for x in (eps, mu))
+            YT = mtp.mtp_evolve_autograd(Y, pe, pm, t, every)
+            if name == "ball32" and prec == mtp.MTP_FP64:    # patch beyond the adjoint's shared memory: refused
+                with pytest.raises(mtp.MtpError, match="shared memory"):
+                    torch.autograd.grad(0.5 * YT.square().sum(), (Y, pe, pm))
+                continue
+            gY, ge, gm = torch.autograd.grad(0.5 * YT.square().sum(), (Y, pe, pm))
+            got = [(gY.double() * dY).sum().item(), (ge.cpu().numpy() * de).sum(), (gm.cpu().numpy() * dm).sum()]
+            for a, b in zip(got, want):
+                assert abs(a - b) <= tol * scale, (prec, every, got, want)
