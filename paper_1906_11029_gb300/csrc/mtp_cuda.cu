@@ -407,7 +407,7 @@ int device_mesh_upload(Mesh& m) {
                     }
             MTP_TRY(upload(&d.Dtc, bt.data(), bt.size()));
         }
-        if (m.precision == MTP_FP32) {
+        if (m.precision == MTP_FP32 || (m.precision == MTP_FP32_SPLIT && m.dim == 3 && m.p <= 3)) {
             MTP_TRY(upload_real(m, &d.Mc1, thread_major(m.ref.M, nv, nbm, m.nb, w, 1)));
             MTP_TRY(upload_real(m, &d.Dc1, thread_major(Dt, m.dim, m.nb, nbm, w, 1)));
             MTP_TRY(upload_real(m, &d.Trc1, thread_major(m.ref.Tr, nv, m.nfb, m.nb, w, 1)));
@@ -503,8 +503,23 @@ static int device_tents_upload(Tents& t) {
     return MTP_OK;
 }
 
+// Shape variant of the tents' kernel: the caller's, and in the 3D split mode, which has no variants to
+// choose from, the one that is faster for the layers (the same bits either way).  Shape 2 wins while a
+// layer is at most a CTA per SM and a row of it is short: 60 layers of 143 tents (p = 1, 2, 3) 1.68, 3.75,
+// 10.0 ms with shape 1 against 1.48, 3.38, 9.7 ms; of 240 tents 1.70, 4.34, 13.1 against 2.23, 5.11, 14.4.
+// At p = 4 shape 2 loses everywhere (27 ms against 38 ms).
+static int item_shape(const Tents& t) {
+    const Mesh& m = *t.mesh;
+    if (m.precision != MTP_FP32_SPLIT || m.dim != 3 || m.p > 3) return t.variant;
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return t.variant;
+    const int64_t layers = (int64_t)t.layer_ptr.size() - 1;
+    return (int64_t)t.vertex.size() <= nsm * layers ? 2 : t.variant;
+}
+
 static const KernelEntry& kernel_entry(const Mesh& m, int variant = 0) {
-    static KernelEntry f64[2][5], f32[2][5], tc[2][5], split[2][5], rk4[2][5], f32v1[2][5], f32v2[2][5], tc5[2][5];
+    static KernelEntry f64[2][5], f32[2][5], tc[2][5], split[2][5], narrow[3], rk4[2][5], f32v1[2][5], f32v2[2][5], tc5[2][5];
     static bool init = false;
     if (!init) {
         kernel_table_f32_tc5(tc5);
@@ -512,6 +527,7 @@ static const KernelEntry& kernel_entry(const Mesh& m, int variant = 0) {
         kernel_table_f32(f32);
         kernel_table_tc(tc);
         kernel_table_split(split);
+        kernel_table_split_narrow(narrow);
         kernel_table_rk4(rk4);
         kernel_table_f32_v1(f32v1);
         kernel_table_f32_v2(f32v2);
@@ -524,6 +540,7 @@ static const KernelEntry& kernel_entry(const Mesh& m, int variant = 0) {
     if (variant == 1 && m.precision == MTP_FP32 && !(m.flags & MTP_FLAG_SUBSTITUTED_RK4))
         return f32v1[m.dim - 2][m.p - 1];
     if (m.flags & MTP_FLAG_SUBSTITUTED_RK4) return rk4[m.dim - 2][m.p - 1];   // FP64 only (checked at creation)
+    if (m.precision == MTP_FP32_SPLIT && variant == 2) return narrow[m.p - 1];
     if (m.precision == MTP_FP32_SPLIT) return split[m.dim - 2][m.p - 1];
     if (m.precision == MTP_TF32 || m.precision == MTP_TF32X3)
         return tc[m.precision == MTP_TF32 ? 0 : 1][m.p - 1];
@@ -558,7 +575,8 @@ static void fill_args(Tents& t, void* state, KArgs& a) {
     a.Dc = dm.Dc;
     a.Trc = dm.Trc;
     a.Lc = dm.Lc;
-    if (t.variant == 2 || t.variant == 4) {   // one row per thread: one row group per matrix row
+    const int shape = item_shape(t);
+    if (shape == 2 || shape == 4) {   // one row per thread: one row group per matrix row
         a.Mc = dm.Mc1;
         a.Dc = dm.Dc1;
         a.Trc = dm.Trc1;
@@ -589,7 +607,7 @@ static void fill_args(Tents& t, void* state, KArgs& a) {
 }
 
 static int enqueue_layers(Tents& t, const KArgs& a, int64_t lb, int64_t le, cudaStream_t st) {
-    const KernelEntry& ke = kernel_entry(*t.mesh, t.variant);
+    const KernelEntry& ke = kernel_entry(*t.mesh, item_shape(t));
     for (int64_t l = lb; l < le; ++l) {
         const int64_t t0 = t.layer_ptr[l];
         const int64_t n = t.layer_ptr[l + 1] - t0;
@@ -624,7 +642,7 @@ int device_evolve(Tents& t, void* state, int64_t lb, int64_t le, bool use_graph,
     Mesh& m = *t.mesh;
     DeviceTents& d = *t.dev;
     cudaStream_t st = (cudaStream_t)stream;
-    const KernelEntry& ke = kernel_entry(m, t.variant);
+    const KernelEntry& ke = kernel_entry(m, item_shape(t));
     size_t smem = 0;
     const cudaError_t pe = ke.prepare(m.max_patch, &smem);
     int dev, smem_max;
@@ -779,7 +797,7 @@ int device_adjoint(Tents& t, const void* state0, const void* lamT, void* lam0, d
     if (m.precision == MTP_FP32_SPLIT || (m.flags & MTP_FLAG_SUBSTITUTED_RK4))
         return set_error(MTP_EUNSUPPORTED, "the adjoint runs SAT meshes in FP64, FP32 or a tensor-core mode");
     const AdjEntry& ae = table[m.precision == MTP_FP64 ? 0 : 1][m.dim - 2][m.p - 1];
-    const KernelEntry& ke = kernel_entry(m, t.variant);
+    const KernelEntry& ke = kernel_entry(m, item_shape(t));
     size_t smem = 0, smem_f = 0;
     const cudaError_t pa_ = ae.prepare(m.max_patch, &smem);
     const cudaError_t pf_ = ke.prepare(m.max_patch, &smem_f);

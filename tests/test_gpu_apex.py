@@ -202,3 +202,29 @@ def test_apex_adjoint_matches_directional_differences(name, p):
             got = [(gY.double() * dY).sum().item(), (ge.cpu().numpy() * de).sum(), (gm.cpu().numpy() * dm).sum()]
             for a, b in zip(got, want):
                 assert abs(a - b) <= tol * scale, (prec, every, got, want)
+
+
+@pytest.mark.parametrize("n,p,wide", [(2, 1, 0), (3, 2, 0), (2, 3, 0), (22, 1, 1), (22, 2, 1), (22, 3, 1), (2, 4, 0), (2, 5, 0)])
+def test_split_shapes_match_fp64(n, p, wide):
+    """Split precision on both sides of the layer-width rule against FP64 (FP32 operator: 1e-5), and the
+    persistent walk against per-layer launches (the same bits)."""
+    v, e = S.cube_mesh(n)
+    x = 2.0 ** (3 * v) / 8       # graded, so that layers are wide
+    eps = 1 + np.random.default_rng(n).random(len(e))
+    outs = []
+    for prec in (mtp.MTP_FP64, mtp.MTP_FP32_SPLIT):
+        if prec == mtp.MTP_FP64 and p == 5:
+            prec = mtp.MTP_FP32     # FP64 has no p = 5 in 3D
+        m = mtp.Mesh(3, x if wide else v, e, eps, np.ones(len(e)), p=p, precision=prec)
+        t = m.pitch(0.002 if wide else 0.1, 0.5)
+        ptr = t.get()["layer_ptr"]
+        assert (ptr[-1] > 152 * (len(ptr) - 1)) == bool(wide)
+        Y0 = torch.tensor(np.random.default_rng(p).standard_normal(m.state_shape), device=DEV)
+        Y = Y0.to(m.torch_dtype(), copy=True)
+        t.evolve(Y)
+        outs.append(Y.double())
+    Z = Y0.clone()
+    t.set_launch(2)
+    t.evolve(Z)
+    assert torch.equal(Z, outs[1])
+    assert ((outs[0] - outs[1]).norm() / outs[0].norm()).item() < 1e-5
