@@ -34,7 +34,8 @@ import hashlib  # noqa: E402
 import numpy as np  # noqa: E402
 
 FP32_SM_LANES = 128            # FP32 FMA lanes per SM (Blackwell)
-KERNEL_SOURCES = ["paper_1906_11029_gb300/csrc/mtp_kernels.cuh", "paper_1906_11029_gb300/csrc/mtp_launch.cuh"]
+KERNEL_SOURCES = ["paper_1906_11029_gb300/csrc/mtp_kernels.cuh", "paper_1906_11029_gb300/csrc/mtp_launch.cuh",
+                  "paper_1906_11029_gb300/csrc/mtp_apex.cuh", "paper_1906_11029_gb300/csrc/mtp_apexgen.cpp"]
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per tent of the tent kernels on the
 # graded 32^3 workload, from an ncu capture of a window of layers (scaled per tent), keyed by
 # (precision, kernel) and stamped with the hash of the kernel sources at capture time: a
@@ -45,6 +46,14 @@ TRAFFIC_BYTES_PER_TENT = {
     # 1000..1099 (81 105 tents) of the graded 32^3 p = 4 workload: 1.145 GB + 0.757 GB
     ("fp32", "tent_persistent_kernel"): {"bytes_per_tent": 23455.2, "sources": "215962c12a1e8c1c"},
 }
+
+
+def tent_kernel_name(precision, variant, dim, p, persistent):
+    """The tent kernel that an evolve launches: apex kernels for FP32 and FP64 in 2D and in 3D up to p = 4."""
+    form = "persistent_kernel" if persistent else "layer_kernel"
+    if precision in ("fp32", "fp64") and variant <= 2 and (dim == 2 or p <= 4):
+        return ("apex2_" if dim == 2 else "apex_") + form
+    return "tent_" + form
 
 
 def kernel_source_hash():
@@ -276,7 +285,7 @@ def run_profile(args):
     torch.cuda.synchronize()
     launches = int(np.count_nonzero(np.diff(tents.get()["layer_ptr"][a:b + 1]))) if args.layer_launches else 1
     print(json.dumps({"profile_window": [a, b], "launches": launches, "workload": w.name,
-                      "kernel": "tent_layer_kernel" if args.layer_launches else "tent_persistent_kernel"}))
+                      "kernel": tent_kernel_name(args.precision, args.variant, w.dim, w.p, not args.layer_launches)}))
 
 
 def run_profile_evolve(args):
@@ -585,7 +594,7 @@ def run_mtp(args):
     else:
         peak, src = probe["fp64_fma"], "mtp_probe_rates FP64 FMA loop on this device, this run"
     achieved = flops_per_launch / (launch_ms / 1e3) / 1e12
-    kname = "tent_persistent_kernel" if persistent else "tent_layer_kernel"
+    kname = tent_kernel_name(args.precision, args.variant, w.dim, w.p, persistent)
     # the stored traffic is the default kernel's (variant 0, occupancy-limit DAG walk)
     default_kernel = args.variant == 0 and args.launch == 0
     tpl = traffic_per_tent(args.precision, kname) if args.workload == "graded" and default_kernel else None

@@ -9,7 +9,8 @@
 // barrier ends a round (its last arriver decides whether the rounds go on).  A block appends its
 // tents to a list of its own; after kPitchChunk rounds two kernels order the lists by (round,
 // block), which is (round, vertex) since blocks own ascending ranges.  (Three kernels a round
-// took 37 us a round on a mesh of 4913 vertices, launches and their gaps for the most part.)
+// took 37 us a round on a mesh of 4913 vertices, launches and their gaps for the most part;
+// now 16 us, the barrier and dependent loads: 62 -> 26 ms for its 1644 rounds.)
 //
 // Layer = round: if V is selected in round r and no vertex of {V} u N(V) moved in round r - 1, V's
 // test gave the same answer in round r - 1 and V would have moved then; so some vertex of the closed
