@@ -242,13 +242,6 @@ void emit_lattice(FILE* f, int d, int p) {
         }
         std::fprintf(f, "        put(%d, %s);\n", a, s.c_str());
     }
-    // every entry, in the order of the points
-    std::fprintf(f, "    }\n    template <typename Put>\n    static __device__ __forceinline__ void from_dense(const double* v, Put put) {\n");
-    for (int a = 0; a < nb; ++a) {
-        std::string s = lit(t.Vinv[(size_t)a * nb]) + " * v[0]";
-        for (int k = 1; k < nb; ++k) s = "__fma_rn(" + lit(t.Vinv[(size_t)a * nb + k]) + ", v[" + std::to_string(k) + "], " + s + ")";
-        std::fprintf(f, "        put(%d, %s);\n", a, s.c_str());
-    }
     std::fprintf(f, "    }\n};\n\n");
 }
 

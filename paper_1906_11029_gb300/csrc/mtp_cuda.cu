@@ -30,6 +30,7 @@ struct DeviceMesh {
     void* Dc = nullptr;
     void* Trc = nullptr;
     void* Lc = nullptr;
+    double* lattice[2] = {nullptr, nullptr};   // V and its inverse
     void* Mc1 = nullptr;          // the same four tables with one row per thread (shape variant 2)
     void* Dc1 = nullptr;
     void* Trc1 = nullptr;
@@ -369,6 +370,8 @@ int device_mesh_upload(Mesh& m) {
     DeviceMesh& d = *m.dev;
     d.device = dev;
     MTP_TRY(upload(&d.geo, m.geo.data(), m.geo.size()));
+    MTP_TRY(upload(&d.lattice[0], m.ref.V.data(), m.ref.V.size()));
+    MTP_TRY(upload(&d.lattice[1], m.ref.Vinv.data(), m.ref.Vinv.size()));
     MTP_TRY(upload(&d.elems, m.elems.data(), m.elems.size()));
     MTP_TRY(upload(&d.patch_ptr, m.patch_ptr.data(), m.patch_ptr.size()));
     MTP_TRY(upload(&d.patch_elem, m.patch_elem.data(), m.patch_elem.size()));
@@ -448,7 +451,7 @@ int device_mesh_upload(Mesh& m) {
 void device_mesh_free(Mesh& m) {
     if (!m.dev) return;
     DeviceMesh& d = *m.dev;
-    void* ptrs[] = {d.geo, d.elems, d.patch_ptr, d.patch_elem, d.patch_info, d.S, d.Tr, d.L, d.Mc, d.Dc, d.Trc, d.Lc, d.Mc1, d.Dc1, d.Trc1, d.Lc1,
+    void* ptrs[] = {d.lattice[0], d.lattice[1], d.geo, d.elems, d.patch_ptr, d.patch_elem, d.patch_info, d.S, d.Tr, d.L, d.Mc, d.Dc, d.Trc, d.Lc, d.Mc1, d.Dc1, d.Trc1, d.Lc1,
                     d.partial,
                     d.Sf, d.Lfr, d.Trf, d.Sf_lo, d.Lfr_lo, d.Trf_lo, d.Dtc, d.ent, d.Rt, d.apex2};
     for (void* p : ptrs)
@@ -549,6 +552,7 @@ static const KernelEntry& kernel_entry(const Mesh& m, int variant = 0) {
 
 
 const double* device_geo(const Mesh& m) { return m.dev->geo; }
+const double* const* device_lattice_tables(const Mesh& m) { return m.dev->lattice; }
 double* device_energy_scratch(const Mesh& m) { return m.dev->partial; }
 
 // ---------------------------------------------------------------------------------

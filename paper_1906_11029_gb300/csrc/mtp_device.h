@@ -29,6 +29,7 @@ inline bool state_f64(const Mesh& m) { return m.precision == MTP_FP64 || m.preci
 
 // device copies that belong to an uploaded mesh (mtp_cuda.cu)
 const double* device_geo(const Mesh& m);
+const double* const* device_lattice_tables(const Mesh& m);   // V and its inverse
 double* device_energy_scratch(const Mesh& m);
 // doubles that device_energy_scratch holds (mtp_lattice.cu)
 size_t energy_scratch_doubles(const Mesh& m);

@@ -57,9 +57,7 @@ __global__ void __launch_bounds__(LatShape<DIM, P>::NT) to_lattice_kernel(const 
     }
 }
 
-// DENSE: the products in the order of the points.  A split-precision evolve turns a change in the last
-// bit of its FP64 state into one of its FP32 arithmetic, so its states keep this order.
-template <typename Real, int DIM, int P, bool DENSE>
+template <typename Real, int DIM, int P>
 __global__ void __launch_bounds__(LatShape<DIM, P>::NT) from_lattice_kernel(const double* vals, Real* state, const double* geo,
                                                                             int64_t ne, int64_t n) {
     using Sh = LatShape<DIM, P>;
@@ -80,12 +78,64 @@ __global__ void __launch_bounds__(LatShape<DIM, P>::NT) from_lattice_kernel(cons
         const double sq = 1.0 / geo[(e0 + k) % ne * kGeoStride + 28];
         __syncthreads();
         auto put = [&](int a, double y) { out[lane * SP + f * NB + a] = (Real)(sq * y); };
-        if constexpr (DENSE) LatticeOps<DIM, P>::from_dense(v, put);
-        else LatticeOps<DIM, P>::from(v, put);
+        LatticeOps<DIM, P>::from(v, put);
         __syncthreads();
         Real* dst = state + e0 * NC;
         for (int i = threadIdx.x; i < ns * NC; i += NT) dst[i] = out[i / NC * SP + i % NC];
         __syncthreads();
+    }
+}
+
+// Few elements: a thread per value with the dense products, in the order of the points or functions, which
+// spreads them over all SMs.  The kernels above take as long for one CTA as for one on every SM: in FP32
+// at degree 4, 45 / 55 us to / from the lattice with 96 CTAs (3072 elements); these take 17 / 24 us for 384
+// elements, of which 14 / 23 us are the call.
+template <typename Real>
+__global__ void __launch_bounds__(128) to_lattice_small_kernel(const Real* state, double* vals, const double* geo, const double* V,
+                                                               int64_t ne, int nf, int nb, int64_t n) {
+    const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    if (i >= n) return;
+    const int64_t ek = i / nf, e = ek / nb;
+    const int f = (int)(i - ek * nf), k = (int)(ek - e * nb);
+    const Real* x = state + (e * nf + f) * nb;
+    double acc = 0;
+#pragma unroll 8
+    for (int a = 0; a < nb; ++a) acc += V[k * nb + a] * (double)x[a];
+    vals[i] = geo[e % ne * kGeoStride + 28] * acc;
+}
+
+template <typename Real>
+__global__ void __launch_bounds__(128) from_lattice_small_kernel(const double* vals, Real* state, const double* geo,
+                                                                 const double* Vinv, int64_t ne, int nf, int nb, int64_t n) {
+    const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    if (i >= n) return;
+    const int64_t ef = i / nb, e = ef / nf;
+    const int a = (int)(i - ef * nb), f = (int)(ef - e * nf);
+    const double* v = vals + e * nb * nf + f;
+    const double sq = 1.0 / geo[e % ne * kGeoStride + 28];
+    double acc = 0;
+#pragma unroll 8
+    for (int k = 0; k < nb; ++k) acc += Vinv[a * nb + k] * v[k * nf];
+    state[i] = (Real)(sq * acc);
+}
+
+// DENSE states of many elements: a thread per (element, function), products in the order of the points.  A
+// split-precision evolve turns a change in the last bit of its FP64 state into one of its FP32
+// arithmetic, so its states keep this order.  (34 992 elements of degree 4: 465 us; a warp per field with the
+// dense products in registers takes 582 us, a thread per value 513 us.)
+template <typename Real>
+__global__ void __launch_bounds__(256) from_lattice_dense_kernel(const double* vals, Real* state, const double* geo,
+                                                                 const double* Vinv, int64_t ne, int nf, int nb, int64_t n) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = i / nb;
+        const int a = (int)(i - e * nb);
+        const double sq = 1.0 / geo[e % ne * kGeoStride + 28];
+        const double* v = vals + e * nb * nf;
+        for (int f = 0; f < nf; ++f) {
+            double acc = 0;
+            for (int k = 0; k < nb; ++k) acc += Vinv[a * nb + k] * v[k * nf + f];
+            state[(e * nf + f) * nb + a] = (Real)(sq * acc);
+        }
     }
 }
 
@@ -153,6 +203,11 @@ int lattice_grid(int64_t n) {
     return (int)(g < 152 * 32 ? g : 152 * 32);
 }
 
+// Elements up to which the small kernels run: while the others leave half of the SMs without a CTA.  There the
+// two take the same time (2058 elements of degree 4, FP32, to the lattice: 64 us with the small kernel, 3072
+// elements 91 us with it and 45 us with the other).
+constexpr int64_t kSmallElems = 16 * 152;
+
 template <typename K>
 cudaError_t lattice_smem(K kernel, size_t bytes) {
     return bytes > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) : cudaSuccess;
@@ -164,6 +219,11 @@ struct Lattice {
     static cudaError_t to(const Mesh& m, const void* state, double* vals, cudaStream_t st) {
         constexpr size_t bytes = (size_t)kLatElems * Sh::SP * sizeof(double);
         const int64_t n = (int64_t)m.n_rhs * m.ne;
+        if (n <= kSmallElems) {
+            to_lattice_small_kernel<Real><<<(unsigned)((n * Sh::NC + 127) / 128), 128, 0, st>>>(
+                (const Real*)state, vals, device_geo(m), device_lattice_tables(m)[0], m.ne, Sh::NF, Sh::NB, n * Sh::NC);
+            return cudaGetLastError();
+        }
         const cudaError_t e = lattice_smem(to_lattice_kernel<Real, DIM, P>, bytes);
         if (e != cudaSuccess) return e;
         to_lattice_kernel<Real, DIM, P><<<lattice_grid(n), Sh::NT, bytes, st>>>((const Real*)state, vals, device_geo(m), m.ne, n);
@@ -172,9 +232,20 @@ struct Lattice {
     static cudaError_t from(const Mesh& m, const double* vals, void* state, cudaStream_t st) {
         constexpr size_t bytes = (size_t)kLatElems * Sh::SP * sizeof(double);
         const int64_t n = (int64_t)m.n_rhs * m.ne;
-        const cudaError_t e = lattice_smem(from_lattice_kernel<Real, DIM, P, DENSE>, bytes);
-        if (e != cudaSuccess) return e;
-        from_lattice_kernel<Real, DIM, P, DENSE><<<lattice_grid(n), Sh::NT, bytes, st>>>(vals, (Real*)state, device_geo(m), m.ne, n);
+        if (n <= kSmallElems) {
+            from_lattice_small_kernel<Real><<<(unsigned)((n * Sh::NC + 127) / 128), 128, 0, st>>>(
+                vals, (Real*)state, device_geo(m), device_lattice_tables(m)[1], m.ne, Sh::NF, Sh::NB, n * Sh::NC);
+            return cudaGetLastError();
+        }
+        if constexpr (DENSE) {
+            const int64_t rows = n * Sh::NB, g = (rows + 255) / 256;
+            from_lattice_dense_kernel<Real><<<(unsigned)(g < 65535 ? g : 65535), 256, 0, st>>>(
+                vals, (Real*)state, device_geo(m), device_lattice_tables(m)[1], m.ne, Sh::NF, Sh::NB, rows);
+        } else {
+            const cudaError_t e = lattice_smem(from_lattice_kernel<Real, DIM, P>, bytes);
+            if (e != cudaSuccess) return e;
+            from_lattice_kernel<Real, DIM, P><<<lattice_grid(n), Sh::NT, bytes, st>>>(vals, (Real*)state, device_geo(m), m.ne, n);
+        }
         return cudaGetLastError();
     }
     static cudaError_t energy(const Mesh& m, const void* state, double* partial, cudaStream_t st) {

@@ -147,6 +147,25 @@ def test_lattice_exchange_and_energy(dim, p):
 
 
 @pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5])
+def test_lattice_exchange_many_elements(dim, p):
+    """More elements (over all right-hand sides) than the small kernels take, not a multiple of 32, against one
+    right-hand side at a time, which they do take: 1e-13 in FP64, an FP32 rounding for an FP32 state, the same
+    bits for split precision (products in one order)."""
+    v, e = S.square_mesh(27) if dim == 2 else S.cube_mesh(5)
+    one, nrhs = np.ones(len(e)), 2 if dim == 2 else 4
+    for prec, tol in ((mtp.MTP_FP64, 1e-13), (mtp.MTP_FP32, 2.0 ** -23), (mtp.MTP_FP32_SPLIT, 0.0)):
+        many = mtp.Mesh(dim, v, e, one, one, p=p, precision=prec, n_rhs=nrhs)
+        few = mtp.Mesh(dim, v, e, one, one, p=p, precision=prec)
+        nf, nb = many.state_shape[-2:]
+        vals = torch.tensor(np.random.default_rng(p).standard_normal((nrhs, len(e), nb, nf)), device=DEV)
+        st, want = many.state_from_lattice(vals), torch.cat([few.state_from_lattice(x[None].contiguous()) for x in vals])
+        assert (st - want).norm().item() <= tol * want.norm().item()
+        back, want = many.state_to_lattice(st), torch.cat([few.state_to_lattice(x[None].contiguous()) for x in st])
+        assert (back - want).norm().item() <= 1e-13 * want.norm().item()
+
+
+@pytest.mark.parametrize("dim", [2, 3])
 def test_vertex_without_elements(dim):
     """A vertex that no element uses has a tent of no elements; the rest of the mesh is not affected."""
     v, e = S.square_mesh(2) if dim == 2 else S.cube_mesh(1)
