@@ -558,7 +558,9 @@ double* device_energy_scratch(const Mesh& m) { return m.dev->partial; }
 // ---------------------------------------------------------------------------------
 // evolution
 // ---------------------------------------------------------------------------------
-static void fill_args(Tents& t, void* state, KArgs& a) {
+// `shape`: the item shape of the kernel that reads the arguments, which decides the row grouping of its
+// thread-major tables (general batch and adjoint kernels: 0 whatever variant the handle has)
+static void fill_args(Tents& t, void* state, KArgs& a, int shape) {
     Mesh& m = *t.mesh;
     DeviceMesh& dm = *m.dev;
     DeviceTents& dt = *t.dev;
@@ -579,7 +581,6 @@ static void fill_args(Tents& t, void* state, KArgs& a) {
     a.Dc = dm.Dc;
     a.Trc = dm.Trc;
     a.Lc = dm.Lc;
-    const int shape = item_shape(t);
     if (shape == 2 || shape == 4) {   // one row per thread: one row group per matrix row
         a.Mc = dm.Mc1;
         a.Dc = dm.Dc1;
@@ -660,7 +661,7 @@ int device_evolve(Tents& t, void* state, int64_t lb, int64_t le, bool use_graph,
     MTP_TRY(set_front(t, lb, d.tau, st));
     CUDA_TRY(cudaMemsetAsync(d.err, 0, sizeof(int), st));
     KArgs a;
-    fill_args(t, state, a);
+    fill_args(t, state, a, item_shape(t));
     const bool full = lb == 0 && le == (int64_t)t.layer_ptr.size() - 1;
     const int launch = (m.flags & MTP_FLAG_LAYER_LAUNCHES) ? 2 : t.launch;
     if (launch != 2 && le > lb) {
@@ -866,7 +867,7 @@ int device_adjoint(Tents& t, const void* state0, const void* lamT, void* lam0, d
     for (int64_t c = 0; c < nck; ++c) {
         CUDA_TRY(cudaMemcpyAsync(ckpt(c), work, sbytes, cudaMemcpyDeviceToDevice, st));
         if (c + 1 == nck) break;   // the last segment's layers run when it is reversed
-        fill_args(t, work, fa);
+        fill_args(t, work, fa, item_shape(t));
         MTP_TRY(enqueue_layers(t, fa, c * K, (c + 1) * K, st));
     }
     // reverse sweep
@@ -884,7 +885,7 @@ int device_adjoint(Tents& t, const void* state0, const void* lamT, void* lam0, d
         const int64_t e0 = off[t.layer_ptr[l0]];
         MTP_TRY(set_front(t, l0, d.tau, st));
         CUDA_TRY(cudaMemcpyAsync(work, ckpt(c), sbytes, cudaMemcpyDeviceToDevice, st));
-        fill_args(t, work, fa);
+        fill_args(t, work, fa, item_shape(t));
         for (int64_t l = l0; l < l1; ++l) {
             MTP_TRY(patch_tape(t, work, ptape, l, e0, seg_entries, true, st));
             if (l + 1 < l1) MTP_TRY(enqueue_layers(t, fa, l, l + 1, st));
@@ -893,7 +894,7 @@ int device_adjoint(Tents& t, const void* state0, const void* lamT, void* lam0, d
             const int64_t t0 = t.layer_ptr[l], n = t.layer_ptr[l + 1] - t0;
             if (n == 0) continue;
             MTP_TRY(patch_tape(t, ybot, ptape, l, e0, seg_entries, false, st));
-            fill_args(t, nullptr, aa.k);
+            fill_args(t, nullptr, aa.k, 0);
             aa.k.tau = d.tau_rev;
             aa.ybot = ybot;
             aa.lam = lam0;
@@ -974,7 +975,7 @@ int device_batch_evolve(Batch& b, void* const* states, void* stream) {
         Tents& t = *b.inst[i];
         Mesh& m = *t.mesh;
         smem = std::max(smem, be.smem_bytes(m.p, m.max_patch));
-        fill_args(t, states[i], ka[i]);
+        fill_args(t, states[i], ka[i], 0);
         ka[i].err = d.err;
         DeviceTents& dt = *t.dev;
         pa[i].n_tents = (int64_t)t.vertex.size();
