@@ -62,7 +62,8 @@ extern "C" {
 
 /* precision of the state and of the operator arithmetic */
 #define MTP_FP64   0   /* FP64 state and arithmetic */
-#define MTP_FP32   1   /* FP32 state and arithmetic (element geometry and causality test in FP64) */
+#define MTP_FP32   1   /* FP32 state and arithmetic; element geometry is computed and the causality test made
+                          in FP64, the geometry that a tent uses is rounded to FP32 */
 #define MTP_TF32   2   /* 3D: FP32 state; traces, volume and lift contractions on tensor cores
                           with TF32 operands and FP32 accumulation */
 #define MTP_TF32X3 3   /* 3D: as MTP_TF32 with each operand split into TF32 hi + lo parts and
@@ -169,12 +170,17 @@ int mtp_evolve(mtp_tents_t tents, void* state_dev, double T, void* stream);
 int mtp_tents_set_launch(mtp_tents_t tents, int launch);
 
 /* Kernel shape variant of this tents handle (MTP_FP32 SAT meshes).  In 2D, and in 3D up to p = 4,
- * variants 0, 1 and 2 all select the apex tent kernel, which is the fastest for every layer width.
- * For 3D p = 5: 0 (default) each stage item of the tent kernel covers a pair of patch elements with
+ * variants 0, 1 and 2 all select the apex tent kernel, which is the fastest for every layer width,
+ * unless the mesh is stretched: with the stretch of an element its longest edge over its smallest
+ * height, where the largest exceeds 12 or the root mean square 7.5 (a regular Kuhn cube has 2.4), FP32
+ * and FP64 meshes run the general tent kernel, whose rounding error does not grow with the stretch
+ * (3D, p = 2, FP32, a cube stretched 10 and 100 times: 3.5e-7 and 3.5e-7; the apex kernel 2.5e-6 and
+ * 2.7e-4); batches with such a mesh and gradients on it likewise.  There, and for 3D p = 5:
+ * 0 (default) each stage item of the tent kernel covers a pair of patch elements with
  * the same local index of the tent vertex, which share every reference-table read; 1 each item
  * covers one element: twice the items at half the work each, so a tent finishes sooner when the
  * layers hold fewer tents than the GPU has CTA slots; 2 each item covers one element and one basis
- * function (or facet mode), with 512 threads per CTA.  3 and 4 (3D, p = 2..4, patches
+ * function (or facet mode), with 512 threads per CTA in 3D.  3 and 4 (3D, p = 2..4, patches
  * of at most 42 tetrahedra): the item shapes of 1 and 2 on 512 threads, with the volume term of
  * the operator (Sec. 3, the element integrals of the DG semi-discretisation) computed on the
  * tcgen05 tensor cores as TF32 MMAs with a three-term hi + lo operand split and FP32

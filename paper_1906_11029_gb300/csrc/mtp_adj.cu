@@ -30,7 +30,7 @@ int64_t adjoint_tape_stride(int max_patch, int m, int q) {
 
 #define ADJ_ENTRY(REAL, D, P) {launch_adjoint_kernel<REAL, D, P>, prepare_adjoint_kernel<REAL, D, P>, adjoint_tape_stride<REAL, D, P>}
 
-// 3D up to kApexMaxDegree: the apex form.  The size that decides about MTP_EUNSUPPORTED stays that of the
+// The apex form (3D).  The size that decides about MTP_EUNSUPPORTED stays that of the
 // general kernel, so the same calls are refused.
 template <typename Real, int P>
 cudaError_t prepare_apex_adjoint(int max_patch, size_t* smem_bytes) {
@@ -53,12 +53,18 @@ int64_t apex_adjoint_tape(int, int m, int q) {
 void adjoint_table(AdjEntry e[2][2][5]) {
     AdjEntry t[2][2][5] = {
         {{ADJ_ENTRY(double, 2, 1), ADJ_ENTRY(double, 2, 2), ADJ_ENTRY(double, 2, 3), ADJ_ENTRY(double, 2, 4), ADJ_ENTRY(double, 2, 5)},
-         {APEX_ADJ(double, 1), APEX_ADJ(double, 2), APEX_ADJ(double, 3), ADJ_ENTRY(double, 3, 4), ADJ_ENTRY(double, 3, 5)}},
+         {ADJ_ENTRY(double, 3, 1), ADJ_ENTRY(double, 3, 2), ADJ_ENTRY(double, 3, 3), ADJ_ENTRY(double, 3, 4), ADJ_ENTRY(double, 3, 5)}},
         {{ADJ_ENTRY(float, 2, 1), ADJ_ENTRY(float, 2, 2), ADJ_ENTRY(float, 2, 3), ADJ_ENTRY(float, 2, 4), ADJ_ENTRY(float, 2, 5)},
-         {APEX_ADJ(float, 1), APEX_ADJ(float, 2), APEX_ADJ(float, 3), APEX_ADJ(float, 4), ADJ_ENTRY(float, 3, 5)}}};
+         {ADJ_ENTRY(float, 3, 1), ADJ_ENTRY(float, 3, 2), ADJ_ENTRY(float, 3, 3), ADJ_ENTRY(float, 3, 4), ADJ_ENTRY(float, 3, 5)}}};
     for (int a = 0; a < 2; ++a)
         for (int b = 0; b < 2; ++b)
             for (int c = 0; c < 5; ++c) e[a][b][c] = t[a][b][c];
+}
+void apex_adjoint_table(AdjEntry e[2][5]) {
+    AdjEntry t[2][5] = {{APEX_ADJ(double, 1), APEX_ADJ(double, 2), APEX_ADJ(double, 3), {}, {}},
+                        {APEX_ADJ(float, 1), APEX_ADJ(float, 2), APEX_ADJ(float, 3), APEX_ADJ(float, 4), {}}};
+    for (int a = 0; a < 2; ++a)
+        for (int c = 0; c < 5; ++c) e[a][c] = t[a][c];
 }
 
 }  // namespace mtp

@@ -15,7 +15,8 @@
 // block); A depends on eps, mu through Z = sqrt(mu/eps) in the fluxes: dJ/dZ from forward-mode
 // dual numbers through the same flux routine, then dZ/deps = -Z/(2 eps), dZ/dmu = Z/(2 mu).
 //
-// This general form serves 2D and 3D degrees beyond the apex kernels'; mtp_apex_adjoint.cuh is the other.
+// This general form serves 2D, 3D degrees beyond the apex kernels' and stretched meshes; mtp_apex_adjoint.cuh is
+// the other.
 #pragma once
 
 #include "mtp_kernels.cuh"

@@ -32,7 +32,8 @@
 // Measured against the general kernel on a GB300, one slab: graded 32^3, p = 4, FP32, 463 -> 137 ms
 // (5.2k instead of 17.3k clocks per tent and stage; 52 % of the issue slots, then waits at the
 // barriers); 16^3 cavity, p = 3, FP32, 333 -> 87 ms; 8^3 cavity, p = 3, FP64, 560 -> 259 ms (FP64
-// issue); 13^3, p = 2, FP32 35.7 -> 9.5 ms.  Error against 64 bits: 3.8e-7 -> 1.3e-7, 1.9e-6 -> 5.4e-7.
+// issue); 13^3, p = 2, FP32 35.7 -> 9.5 ms.  Error against 64 bits of the first two: 3.8e-7 -> 1.3e-7, 1.9e-6 -> 5.4e-7;
+// it grows with the stretch of the elements, and beyond kMaxStretch the general kernel runs.
 #pragma once
 
 #include "mtp_apex_ops.h"

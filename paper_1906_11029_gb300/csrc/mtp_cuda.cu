@@ -521,7 +521,8 @@ static int item_shape(const Tents& t) {
     return (int64_t)t.vertex.size() <= nsm * layers ? 2 : t.variant;
 }
 
-static const KernelEntry& kernel_entry(const Mesh& m, int variant = 0) {
+// general tent kernels
+static const KernelEntry& general_entry(const Mesh& m, int variant) {
     static KernelEntry f64[2][5], f32[2][5], tc[2][5], split[2][5], narrow[3], rk4[2][5], f32v1[2][5], f32v2[2][5], tc5[2][5];
     static bool init = false;
     if (!init) {
@@ -550,6 +551,33 @@ static const KernelEntry& kernel_entry(const Mesh& m, int variant = 0) {
     return (m.precision == MTP_FP64 ? f64 : f32)[m.dim - 2][m.p - 1];
 }
 
+// Whether the mesh's tents run in the apex kernels: the plain SAT modes of their degrees, unless the mesh is
+// stretched.  A stretched mesh whose patches are too large for the general kernel's shared memory (FP64, 3D,
+// p = 4, more than 30 tetrahedra) has no other kernel than the apex one.
+static bool apex_runs(const Mesh& m, int variant) {
+    if ((m.precision != MTP_FP64 && m.precision != MTP_FP32) || (m.flags & MTP_FLAG_SUBSTITUTED_RK4) || variant > 2 ||
+        (m.dim == 3 && m.p > kApexMaxDegree))
+        return false;
+    size_t bytes = 0;
+    return !m.stretched || general_entry(m, variant).prepare(m.max_patch, &bytes) != cudaSuccess;
+}
+
+static const KernelEntry& kernel_entry(const Mesh& m, int variant = 0) {
+    if (!apex_runs(m, variant)) return general_entry(m, variant);
+    static KernelEntry apex[2][2][5];
+    static bool init = false;
+    if (!init) {
+        for (int p = 1; p <= 5; ++p) {
+            apex[0][0][p - 1] = apex2_entry_f64(p);
+            apex[1][0][p - 1] = apex2_entry_f32(p);
+            if (p > kApexMaxDegree) continue;
+            apex[0][1][p - 1] = apex_entry_f64(p);
+            apex[1][1][p - 1] = apex_entry_f32(p);
+        }
+        init = true;
+    }
+    return apex[m.precision == MTP_FP64 ? 0 : 1][m.dim - 2][m.p - 1];
+}
 
 const double* device_geo(const Mesh& m) { return m.dev->geo; }
 const double* const* device_lattice_tables(const Mesh& m) { return m.dev->lattice; }
@@ -796,12 +824,13 @@ int device_adjoint(Tents& t, const void* state0, const void* lamT, void* lam0, d
     Mesh& m = *t.mesh;
     DeviceTents& d = *t.dev;
     cudaStream_t st = (cudaStream_t)stream;
-    static AdjEntry table[2][2][5];
+    static AdjEntry general[2][2][5], apex[2][5];
     static bool init = false;
-    if (!init) { adjoint_table(table); init = true; }
+    if (!init) { adjoint_table(general); apex_adjoint_table(apex); init = true; }
     if (m.precision == MTP_FP32_SPLIT || (m.flags & MTP_FLAG_SUBSTITUTED_RK4))
         return set_error(MTP_EUNSUPPORTED, "the adjoint runs SAT meshes in FP64, FP32 or a tensor-core mode");
-    const AdjEntry& ae = table[m.precision == MTP_FP64 ? 0 : 1][m.dim - 2][m.p - 1];
+    const int fp = m.precision == MTP_FP64 ? 0 : 1;   // the tensor-core modes' adjoint runs in FP32
+    const AdjEntry& ae = m.dim == 3 && apex[fp][m.p - 1].launch && !m.stretched ? apex[fp][m.p - 1] : general[fp][m.dim - 2][m.p - 1];
     const KernelEntry& ke = kernel_entry(m, item_shape(t));
     size_t smem = 0, smem_f = 0;
     const cudaError_t pa_ = ae.prepare(m.max_patch, &smem);
@@ -939,20 +968,33 @@ int device_batch_evolve(Batch& b, void* const* states, void* stream) {
     const int64_t ni = (int64_t)b.inst.size();
     for (Tents* t : b.inst) MTP_TRY(device_tents_upload(*t));
     const Mesh& m0 = *b.inst[0]->mesh;
-    static BatchEntry table[2];
+    static BatchEntry general[2][2];
     static bool init = false;
-    if (!init) { batch_table(table); init = true; }
+    if (!init) { batch_table(general); init = true; }
     for (Tents* t : b.inst)
         if (t->mesh->flags & MTP_FLAG_SUBSTITUTED_RK4)
             return set_error(MTP_EUNSUPPORTED, "batches run SAT meshes; MTP_FLAG_SUBSTITUTED_RK4 is per mesh");
     if (m0.precision == MTP_TF32 || m0.precision == MTP_TF32X3 || m0.precision == MTP_FP32_SPLIT)
         return set_error(MTP_EUNSUPPORTED, "batches run FP64 or FP32 SIMT meshes; tensor-core and split modes are per mesh");
-    int pmax = 0;
-    for (Tents* t : b.inst) pmax = std::max(pmax, t->mesh->p);
+    int dev, smem_max;
+    CUDA_TRY(cudaGetDevice(&dev));
+    CUDA_TRY(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const bool f64 = m0.precision == MTP_FP64;
-    const BatchEntry be = m0.dim == 2              ? (f64 ? apex2_batch_f64() : apex2_batch_f32())
-                          : pmax <= kApexMaxDegree ? (f64 ? apex_batch_f64(pmax) : apex_batch_f32(pmax))
-                                                   : table[f64 ? 0 : 1];
+    auto smem_of = [&](const BatchEntry& e) {
+        size_t n = 0;
+        for (Tents* t : b.inst) n = std::max(n, e.smem_bytes(t->mesh->p, t->mesh->max_patch));
+        return n;
+    };
+    int pmax = 0;
+    bool stretched = false;
+    for (Tents* t : b.inst) {
+        pmax = std::max(pmax, t->mesh->p);
+        stretched |= t->mesh->stretched;
+    }
+    BatchEntry be = general[f64 ? 0 : 1][m0.dim - 2];
+    if ((m0.dim == 2 || pmax <= kApexMaxDegree) && (!stretched || (int64_t)smem_of(be) > smem_max))   // see apex_runs
+        be = m0.dim == 2 ? (f64 ? apex2_batch_f64() : apex2_batch_f32()) : (f64 ? apex_batch_f64(pmax) : apex_batch_f32(pmax));
+    const size_t smem = smem_of(be);
     if (!b.dev) {
         b.dev = new DeviceBatch();
         DeviceBatch& d = *b.dev;
@@ -968,13 +1010,11 @@ int device_batch_evolve(Batch& b, void* const* states, void* stream) {
         CUDA_TRY(cudaMallocHost((void**)&d.err_host, sizeof(int)));
     }
     DeviceBatch& d = *b.dev;
-    size_t smem = 0;
     std::vector<KArgs> ka(ni);
     std::vector<PArgs> pa(ni);
     for (int64_t i = 0; i < ni; ++i) {
         Tents& t = *b.inst[i];
         Mesh& m = *t.mesh;
-        smem = std::max(smem, be.smem_bytes(m.p, m.max_patch));
         fill_args(t, states[i], ka[i], 0);
         ka[i].err = d.err;
         DeviceTents& dt = *t.dev;
@@ -993,9 +1033,7 @@ int device_batch_evolve(Batch& b, void* const* states, void* stream) {
         CUDA_TRY(cudaMemsetAsync(dt.tau, 0, sizeof(double) * m.nv, st));   // flat front t = 0
         CUDA_TRY(cudaMemsetAsync(dt.cnt, 0, sizeof(int) * m.nv, st));
     }
-    int dev, smem_max, bpsm = 0, nsm = 0;
-    CUDA_TRY(cudaGetDevice(&dev));
-    CUDA_TRY(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    int bpsm = 0, nsm = 0;
     if ((int64_t)smem > smem_max)
         return set_error(MTP_EUNSUPPORTED, "batch kernel needs " + std::to_string(smem) +
                                                " bytes of shared memory per block; the device allows " +

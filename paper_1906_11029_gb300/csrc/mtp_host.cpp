@@ -78,6 +78,7 @@ static int build_mesh(int dim, int64_t nv, const double* X, int64_t ne, const in
     }
     // geometry
     m.geo.assign(ne * kGeoStride, 0.0);
+    double stretch_max = 0, stretch_sq = 0;
     for (int64_t e = 0; e < ne; ++e) {
         const int32_t* el = &m.elems[e * nvert];
         double P[4][3] = {};
@@ -120,11 +121,18 @@ static int build_mesh(int dim, int64_t nv, const double* X, int64_t ne, const in
             for (int l = 1; l <= dim; ++l) s += gl[l][c];
             gl[0][c] = -s;
         }
-        double adet = std::fabs(det);
+        double adet = std::fabs(det), edge2 = 0, grad2 = 0;
+        for (int i = 0; i < nvert; ++i)
+            for (int j = 0; j < i; ++j) {
+                double l2 = 0;
+                for (int c = 0; c < dim; ++c) l2 += (P[i][c] - P[j][c]) * (P[i][c] - P[j][c]);
+                edge2 = std::fmax(edge2, l2);
+            }
         for (int i = 0; i < nvert; ++i) {
             double n2 = 0;
             for (int c = 0; c < 3; ++c) n2 += gl[i][c] * gl[i][c];
             double nn = std::sqrt(n2);
+            grad2 = std::fmax(grad2, n2);
             for (int c = 0; c < 3; ++c) {
                 g[3 * i + c] = gl[i][c];
                 g[12 + 3 * i + c] = -gl[i][c] / nn;
@@ -135,7 +143,10 @@ static int build_mesh(int dim, int64_t nv, const double* X, int64_t ne, const in
         g[29] = eps[e];
         g[30] = mu[e];
         g[31] = std::sqrt(mu[e] / eps[e]);
+        stretch_max = std::fmax(stretch_max, std::sqrt(edge2 * grad2));
+        stretch_sq += edge2 * grad2;
     }
+    m.stretched = stretch_max > kMaxStretch || std::sqrt(stretch_sq / (double)ne) > kMaxStretchRms;
     // facets: sort (facet key, element, local facet)
     struct FK { int32_t v[3]; int64_t e; int f; };
     std::vector<FK> keys;

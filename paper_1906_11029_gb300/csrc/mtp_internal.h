@@ -61,6 +61,22 @@ RefTables build_ref_tables(int dim, int p);
 //   [28] 1/sqrt|det J|  [29] eps  [30] mu  [31] Z = sqrt(mu/eps)
 constexpr int kGeoStride = 32;
 
+// Stretch of an element: its longest edge over its smallest height (regular Kuhn cube: 2.4).  The apex kernels
+// hold y and U along the edges from the tent vertex, so their rounding error grows with the stretch, and with
+// its square where all three edges are long; the general kernels' (Cartesian components) does not grow.
+// Error against 64 bits in FP32, random data, general | apex, 3D p = 1, 2, 4 (a GB300, cube of 3^3):
+//   cube in z x 2  (3.1)   1.8e-7 3.4e-7 6.7e-7 | 2.0e-7 2.7e-7 4.0e-7
+//   x 4   (5.6)            1.8e-7 3.5e-7 7.0e-7 | 3.5e-7 4.6e-7 6.7e-7
+//   x 5   (6.9)            1.8e-7 3.5e-7 7.1e-7 | 5.4e-7 6.5e-7 9.1e-7
+//   x 10  (14)             1.8e-7 3.4e-7 7.1e-7 | 2.1e-6 2.5e-6 3.3e-6
+//   x 100 (140)            1.8e-7 3.5e-7 7.3e-7 | 2.3e-4 2.7e-4 3.4e-4
+//   in z / 100 (140)       1.4e-7 2.9e-7 7.2e-7 | 6.1e-6 8.2e-6 1.6e-5
+//   graded 8 : 1, 6^3 (largest 11.5, rms 5.7)  1.7e-7 3.2e-7 6.6e-7 | 3.2e-7 3.8e-7 5.9e-7;
+//   the same with a Gaussian pulse             1.2e-7 2.5e-7 5.7e-7 | 0.9e-7 1.4e-7 1.9e-7
+// in FP64 at x 1000: 4e-11 off for the apex kernel, beyond that mode's contract.  The line keeps the meshes
+// graded 8 : 1 from 3^3 elements on, where smooth data are no less accurate than with the general kernel.
+constexpr double kMaxStretch = 12.0, kMaxStretchRms = 7.5;
+
 struct Mesh {
     int dim = 0, p = 0, q = 0, m = 0, precision = 0, n_rhs = 1, flags = 0;
     int nf = 0, nb = 0, nfb = 0, max_patch = 0;
@@ -79,6 +95,7 @@ struct Mesh {
     std::vector<int8_t> patch_info;    // [n_entries][12]
     std::vector<int64_t> adj_ptr;      // vertex adjacency (CSR, ascending)
     std::vector<int32_t> adj;
+    bool stretched = false;            // beyond kMaxStretch or kMaxStretchRms: the general kernels run
     RefTables ref;
     struct DeviceMesh* dev = nullptr;  // lazily created device copies
 };

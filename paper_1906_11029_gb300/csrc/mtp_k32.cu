@@ -1,9 +1,6 @@
-// FP32 kernel table: the apex tent kernels, and the general one in 3D beyond their degrees.
+// FP32 instantiations of the general tent kernels (geometry and the causality test in FP64): 3D p = 5, and
+// stretched meshes at every degree (see kMaxStretch).
 #include "mtp_launch.cuh"
 namespace mtp {
-void kernel_table_f32(KernelEntry e[2][5]) {
-    for (int p = 1; p <= 5; ++p) e[0][p - 1] = apex2_entry_f32(p);
-    for (int p = 1; p <= 4; ++p) e[1][p - 1] = apex_entry_f32(p);
-    e[1][4] = MTP_KERNEL_ENTRY(float, 3, 5, 0);
+MTP_KERNEL_TABLE(kernel_table_f32, float, 0)
 }
-}  // namespace mtp

@@ -1,9 +1,5 @@
-// FP64 kernel table: the apex tent kernels, and the general one in 3D beyond their degrees.
+// FP64 instantiations of the general tent kernels: 3D p = 5, and stretched meshes at every degree.
 #include "mtp_launch.cuh"
 namespace mtp {
-void kernel_table_f64(KernelEntry e[2][5]) {
-    for (int p = 1; p <= 5; ++p) e[0][p - 1] = apex2_entry_f64(p);
-    for (int p = 1; p <= 4; ++p) e[1][p - 1] = apex_entry_f64(p);
-    e[1][4] = MTP_KERNEL_ENTRY(double, 3, 5, 0);
+MTP_KERNEL_TABLE(kernel_table_f64, double, 0)
 }
-}  // namespace mtp

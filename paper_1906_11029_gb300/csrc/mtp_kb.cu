@@ -1,5 +1,5 @@
 // Instantiations of the general many-instance persistent kernel (all degrees in one kernel), for 3D
-// batches with degrees beyond the apex tent kernel's.
+// batches with degrees beyond the apex tent kernel's and for batches with a stretched mesh.
 #include "mtp_launch.cuh"
 
 namespace mtp {
@@ -31,9 +31,11 @@ size_t batch_smem_bytes(int p, int max_patch) {
     }
 }
 
-void batch_table(BatchEntry e[2]) {
-    e[0] = {launch_batch_kernel<double, 3>, prepare_batch_kernel<double, 3>, batch_smem_bytes<double, 3>};
-    e[1] = {launch_batch_kernel<float, 3>, prepare_batch_kernel<float, 3>, batch_smem_bytes<float, 3>};
+void batch_table(BatchEntry e[2][2]) {
+    e[0][0] = {launch_batch_kernel<double, 2>, prepare_batch_kernel<double, 2>, batch_smem_bytes<double, 2>};
+    e[0][1] = {launch_batch_kernel<double, 3>, prepare_batch_kernel<double, 3>, batch_smem_bytes<double, 3>};
+    e[1][0] = {launch_batch_kernel<float, 2>, prepare_batch_kernel<float, 2>, batch_smem_bytes<float, 2>};
+    e[1][1] = {launch_batch_kernel<float, 3>, prepare_batch_kernel<float, 3>, batch_smem_bytes<float, 3>};
 }
 
 }  // namespace mtp

@@ -5,8 +5,15 @@
 #include "mtp_launch.cuh"
 namespace mtp {
 void kernel_table_f32_v2(KernelEntry e[2][5]) {
-    for (int p = 1; p <= 5; ++p) e[0][p - 1] = apex2_entry_f32(p);
-    for (int p = 1; p <= 4; ++p) e[1][p - 1] = apex_entry_f32(p);
+    e[0][0] = MTP_KERNEL_ENTRY(float, 2, 33, 0);
+    e[0][1] = MTP_KERNEL_ENTRY(float, 2, 34, 0);
+    e[0][2] = MTP_KERNEL_ENTRY(float, 2, 35, 0);
+    e[0][3] = MTP_KERNEL_ENTRY(float, 2, 36, 0);
+    e[0][4] = MTP_KERNEL_ENTRY(float, 2, 37, 0);
+    e[1][0] = MTP_KERNEL_ENTRY(float, 3, 33, 0);
+    e[1][1] = MTP_KERNEL_ENTRY(float, 3, 34, 0);
+    e[1][2] = MTP_KERNEL_ENTRY(float, 3, 35, 0);
+    e[1][3] = MTP_KERNEL_ENTRY(float, 3, 36, 0);
     e[1][4] = MTP_KERNEL_ENTRY(float, 3, 37, 0);
 }
 }  // namespace mtp

@@ -65,7 +65,7 @@ struct KernelEntry {
     PersistentPrepFn persistent_prepare;
 };
 
-// entries[dim - 2][p - 1]
+// general tent kernels: entries[dim - 2][p - 1]
 void kernel_table_f64(KernelEntry entries[2][5]);
 void kernel_table_f32(KernelEntry entries[2][5]);
 // tensor-core modes (3D only): entries[mode - 1][p - 1]
@@ -98,8 +98,10 @@ struct AdjEntry {
     PrepareFn prepare;
     TapeStrideFn tape_stride;
 };
-// entries[precision][dim - 2][p - 1]
+// general adjoint: entries[precision][dim - 2][p - 1]
 void adjoint_table(AdjEntry entries[2][2][5]);
+// apex adjoint, 3D: entries[precision][p - 1], FP64 up to p = 3, FP32 up to p = 4 (null beyond)
+void apex_adjoint_table(AdjEntry entries[2][5]);
 
 using BatchLaunchFn = cudaError_t (*)(const BatchArgs&, int grid, size_t smem, cudaStream_t st);
 using BatchPrepFn = cudaError_t (*)(size_t smem, int* blocks_per_sm);
@@ -109,8 +111,8 @@ struct BatchEntry {
     BatchPrepFn prepare;
     BatchSmemFn smem_bytes;
 };
-// 3D batches with degrees beyond the apex kernel's: entries[precision]
-void batch_table(BatchEntry entries[2]);
+// general batch kernel: entries[precision][dim - 2]
+void batch_table(BatchEntry entries[2][2]);
 // 3D batches whose largest degree is at most kApexMaxDegree
 BatchEntry apex_batch_f32(int pmax);
 BatchEntry apex_batch_f64(int pmax);
