@@ -229,7 +229,8 @@ int mtp_batch_evolve(mtp_batch_t batch, void* const* states_dev, void* stream);
  * (the mass operator g(u) - f(u) grad(phi) and the facet impedances).  Dependence of the
  * initial state or of J on eps, mu is the caller's to add.  The forward pass keeps the state
  * before every checkpoint_every-th layer (0: all layers form one segment when their patch tape
- * takes at most 4 GB, about sqrt(n_layers) otherwise); each segment is
+ * takes at most 4 GB and the work buffers at most half of the free device memory, about
+ * sqrt(n_layers) otherwise); each segment is
  * recomputed from its checkpoint and reversed layer by layer, one CTA per tent, replaying
  * the tent's SAT stages into a device tape.  Device work buffers are owned by the tents
  * handle.  Completion and errors as for mtp_evolve; MTP_EUNSUPPORTED if the adjoint kernel's

@@ -853,33 +853,51 @@ int device_adjoint(Tents& t, const void* state0, const void* lamT, void* lam0, d
     for (size_t i = 0; i < t.vertex.size(); ++i)
         off[i + 1] = off[i] + (m.patch_ptr[t.vertex[i] + 1] - m.patch_ptr[t.vertex[i]]);
     if (!d.tent_off) MTP_TRY(upload(&d.tent_off, off.data(), off.size()));
-    if (K <= 0) {
-        // One segment when the patch tape of the whole evolve stays within kAdjointTape: nothing is
-        // computed twice (adjoint workload 8^3, p = 2: 98 MB).  About sqrt(layers) otherwise, which
-        // balances checkpoints and tape at the price of a second forward pass.
-        constexpr size_t kAdjointTape = (size_t)4 << 30;
-        const size_t whole = (size_t)off.back() * m.n_rhs * m.nf * m.nb * real_size(m);
-        K = whole <= kAdjointTape ? nl : std::max<int64_t>(1, (int64_t)std::ceil(std::sqrt((double)nl)));
-    }
-    K = std::min(K, nl);
-    const int64_t nck = (nl + K - 1) / K;
-    int64_t seg_entries = 0;
-    for (int64_t c = 0; c < nck; ++c) {
-        const int64_t l0 = c * K, l1 = std::min((c + 1) * K, nl);
-        seg_entries = std::max(seg_entries, off[t.layer_ptr[l1]] - off[t.layer_ptr[l0]]);
-    }
-    const size_t ptape_bytes = (size_t)seg_entries * m.n_rhs * m.nf * m.nb * real_size(m);
     const int64_t tstride = ae.tape_stride(m.max_patch, m.m, m.q);
     const size_t tape_bytes = (size_t)max_tents * m.n_rhs * tstride * real_size(m);
     auto align = [](size_t x) { return (x + 255) & ~size_t(255); };
-    const size_t need = align((size_t)(nck + 2) * sbytes) + align(ptape_bytes) + tape_bytes + 256;
-    if (d.adj_bytes < need) {
+    int64_t nck = 0, seg_entries = 0;   // segments of K layers, patch entries of the largest
+    size_t ptape_bytes = 0, need = 0;
+    auto plan = [&](int64_t layers) {
+        K = std::min(layers, nl);
+        nck = (nl + K - 1) / K;
+        seg_entries = 0;
+        for (int64_t c = 0; c < nck; ++c) {
+            const int64_t l0 = c * K, l1 = std::min((c + 1) * K, nl);
+            seg_entries = std::max(seg_entries, off[t.layer_ptr[l1]] - off[t.layer_ptr[l0]]);
+        }
+        ptape_bytes = (size_t)seg_entries * m.n_rhs * m.nf * m.nb * real_size(m);
+        need = align((size_t)(nck + 2) * sbytes) + align(ptape_bytes) + tape_bytes + 256;
+    };
+    auto reserve = [&]() {
+        if (d.adj_bytes >= need) return cudaSuccess;
         if (d.adj_buf) cudaFree(d.adj_buf);
         d.adj_buf = nullptr;
         d.adj_bytes = 0;
-        CUDA_TRY(cudaMalloc(&d.adj_buf, need));
-        d.adj_bytes = need;
+        const cudaError_t e = cudaMalloc(&d.adj_buf, need);
+        if (e == cudaSuccess) d.adj_bytes = need;
+        else d.adj_buf = nullptr;
+        return e;
+    };
+    bool reserved = false;
+    if (K <= 0) {
+        // One segment when the patch tape of the whole evolve stays within kAdjointTape and the buffers take
+        // at most half of the free memory (the handle keeps them, and the caller has its own tensors): nothing is
+        // computed twice (adjoint workload 8^3, p = 2: 98 MB).  About sqrt(layers) otherwise, which
+        // balances checkpoints and tape at the price of a second forward pass.
+        constexpr size_t kAdjointTape = (size_t)4 << 30;
+        plan(nl);
+        size_t free_bytes = 0, total = 0;
+        if (d.adj_bytes < need) CUDA_TRY(cudaMemGetInfo(&free_bytes, &total));
+        if (ptape_bytes <= kAdjointTape && (d.adj_bytes >= need || need <= (free_bytes + d.adj_bytes) / 2)) {
+            reserved = reserve() == cudaSuccess;
+            if (!reserved) cudaGetLastError();   // no room after all
+        }
+        if (!reserved) plan(std::max<int64_t>(1, (int64_t)std::ceil(std::sqrt((double)nl))));
+    } else {
+        plan(K);
     }
+    if (!reserved) CUDA_TRY(reserve());
     if (!d.tau_rev) CUDA_TRY(cudaMalloc((void**)&d.tau_rev, sizeof(double) * m.nv));
     char* base = (char*)d.adj_buf;
     auto ckpt = [&](int64_t c) { return (void*)(base + c * sbytes); };
