@@ -913,7 +913,8 @@ int device_adjoint(Tents& t, const void* state0, const void* lamT, void* lam0, d
     KArgs fa;
     for (int64_t c = 0; c < nck; ++c) {
         CUDA_TRY(cudaMemcpyAsync(ckpt(c), work, sbytes, cudaMemcpyDeviceToDevice, st));
-        if (c + 1 == nck) break;   // the last segment's layers run when it is reversed
+        if (c + 1 == nck) break;   // the last segment's layers run when it is reversed, the last layer of all
+                                   // included: it may be the one that a non-finite value first appears in
         fill_args(t, work, fa, item_shape(t));
         MTP_TRY(enqueue_layers(t, fa, c * K, (c + 1) * K, st));
     }
@@ -935,7 +936,7 @@ int device_adjoint(Tents& t, const void* state0, const void* lamT, void* lam0, d
         fill_args(t, work, fa, item_shape(t));
         for (int64_t l = l0; l < l1; ++l) {
             MTP_TRY(patch_tape(t, work, ptape, l, e0, seg_entries, true, st));
-            if (l + 1 < l1) MTP_TRY(enqueue_layers(t, fa, l, l + 1, st));
+            if (l + 1 < l1 || l1 == nl) MTP_TRY(enqueue_layers(t, fa, l, l + 1, st));
         }
         for (int64_t l = l1 - 1; l >= l0; --l) {
             const int64_t t0 = t.layer_ptr[l], n = t.layer_ptr[l + 1] - t0;

@@ -1,5 +1,5 @@
-"""The default checkpoint plan of the gradient: one segment where there is room, about sqrt(layers) where there is
-not, the same gradients either way."""
+"""The default checkpoint plan of the gradient (one segment where there is room, about sqrt(layers) where there is
+not, the same gradients either way), and its report of a forward evolve that fails in the last layer."""
 import numpy as np
 import pytest
 
@@ -38,3 +38,44 @@ def test_default_plan_falls_back_when_memory_is_short():
         torch.cuda.empty_cache()
     for a, b in zip(*out):     # sums by atomics: their order may differ
         assert (a - b).norm().item() <= 1e-13 * a.norm().item()
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("every", [0, 2])
+def test_overflow_in_the_last_layer_is_reported(dim, every):
+    """The gradient reports a forward evolve that first becomes non-finite in its last layer, as the evolve does.  Such
+    an amplitude exists for some states: the largest one that all layers but the last bear is above that of the whole."""
+    v, e = S.square_mesh(1) if dim == 2 else S.cube_mesh(1)
+    one = np.ones(len(e))
+    mesh = mtp.Mesh(dim, v, e, one, one, p=1, precision=mtp.MTP_FP32)
+    tents = mesh.pitch(0.1, 0.5)
+    nl = tents.info["n_layers"]
+
+    def survives(Y, exponent, layers):
+        Z = Y * 2.0 ** exponent
+        try:
+            tents.evolve_layers(Z, 0, layers)
+        except mtp.MtpError as ex:
+            assert ex.code == mtp.MTP_ENUMERIC
+            return False
+        return True
+
+    def limit(Y, layers):
+        lo, hi = 0.0, 127.0
+        while hi - lo > 0.01:
+            mid = 0.5 * (lo + hi)
+            lo, hi = (mid, hi) if survives(Y, mid, layers) else (lo, mid)
+        return lo, hi
+
+    for seed in range(200):
+        Y = torch.randn(mesh.state_shape, generator=torch.Generator().manual_seed(seed)).to(DEV)
+        a, b = limit(Y, nl)[1], limit(Y, nl - 1)[0]
+        if a < b:
+            break
+    else:
+        pytest.fail("no state overflows in the last layer alone")
+    Z = Y * 2.0 ** b
+    l0, ge, gm = torch.empty_like(Z), *(torch.empty(len(e), dtype=torch.float64, device=DEV) for _ in range(2))
+    with pytest.raises(mtp.MtpError) as ex:
+        mtp.mtp_adjoint(tents.h, Z, torch.zeros_like(Z), l0, ge, gm, every)
+    assert ex.value.code == mtp.MTP_ENUMERIC
