@@ -125,8 +125,8 @@ int mtp_pitch_tents(mtp_mesh_t mesh, const double* wavespeed, double causality_f
  * tent's layer equals its round, so the list comes out sorted by (layer, vertex)).
  * The per-edge bounds are computed on the host as in mtp_pitch_tents; the rounds run on
  * `stream`, and the call returns when the tent list is on the host.  Device memory: about
- * 70 bytes per vertex plus 24 bytes per tent of output, allocated and freed inside the
- * call.  MTP_ECUDA / MTP_ENOMEM on CUDA failures. */
+ * 280 bytes per vertex (at least 256 vertices) plus 12 bytes per directed mesh edge, whatever the
+ * number of tents, allocated and freed inside the call.  MTP_ECUDA / MTP_ENOMEM on CUDA failures. */
 int mtp_pitch_tents_device(mtp_mesh_t mesh, const double* wavespeed, double causality_factor,
                            double T, mtp_tents_t* out, void* stream);
 void mtp_tents_destroy(mtp_tents_t tents);

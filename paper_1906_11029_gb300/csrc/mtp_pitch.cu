@@ -7,8 +7,8 @@
 // thousands of rounds with little work each, so they run inside one cooperative kernel: a block
 // owns a contiguous range of vertices, tau is double-buffered by the round's parity, and one grid
 // barrier ends a round (its last arriver decides whether the rounds go on).  A block appends its
-// tents to a list of its own; after kPitchChunk rounds two kernels order the lists by (round,
-// block), which is (round, vertex) since blocks own ascending ranges.  (Three kernels a round
+// tents to a list of its own; after kPitchChunk rounds, or when a list is full, two kernels order the
+// lists by (round, block), which is (round, vertex) since blocks own ascending ranges.  (Three kernels a round
 // took 37 us a round on a mesh of 4913 vertices, launches and their gaps for the most part;
 // now 16 us, the barrier and dependent loads: 62 -> 26 ms for its 1644 rounds.)
 //
@@ -29,6 +29,10 @@ namespace mtp {
 
 constexpr int kPitchThreads = 256;
 constexpr int kPitchChunk = 128;              // rounds per launch at most
+// List entries of a block per vertex it owns.  A round adds at most one a vertex, and the launch ends early when a
+// block's list has no room for another round; usual meshes add 2 .. 5 % of the vertices a round, so that
+// the lists (two of them, 20 bytes an entry) hold a launch's 128 rounds in 240 bytes a vertex.
+constexpr int kPitchList = 6;
 constexpr long long kPitchMaxRounds = 50000000;
 
 struct PitchCtl {
@@ -36,7 +40,8 @@ struct PitchCtl {
     unsigned released;          // rounds whose barrier is open
     int selected;               // vertices selected in the round
     int left;                   // vertices with tau < T
-    int stop;                   // 1 all at T, 2 a round selected nothing, 3 a barrier wait expired
+    int full;                   // a block's list has no room for another round
+    int stop;                   // 1 all at T, 2 a round selected nothing, 3 a barrier wait expired, 4 full
     int rounds;                 // rounds done by the launch
 };
 
@@ -123,6 +128,7 @@ __global__ void __launch_bounds__(kPitchThreads) pitch_rounds_kernel(const Pitch
             const int n = (int)(len - before);
             p.cnt[(int64_t)r * gridDim.x + blockIdx.x] = n;
             if (n) atomicAdd(&p.ctl->selected, n);
+            if (len + p.vpb > p.cap) atomicExch(&p.ctl->full, 1);
             __threadfence();
             if (atomicAdd(&p.ctl->arrived, 1u) == (unsigned)(r + 1) * gridDim.x - 1) {
                 // all blocks are here: their counts are visible, none runs on before the release
@@ -130,6 +136,7 @@ __global__ void __launch_bounds__(kPitchThreads) pitch_rounds_kernel(const Pitch
                 const int left = *(volatile int*)&p.ctl->left, sel = *(volatile int*)&p.ctl->selected;
                 if (left == 0) p.ctl->stop = 1;
                 else if (sel == 0) p.ctl->stop = 2;
+                else if (*(volatile int*)&p.ctl->full) p.ctl->stop = 4;
                 p.ctl->selected = 0;
                 p.ctl->rounds = r + 1;
                 __threadfence();
@@ -249,9 +256,8 @@ int device_pitch(const Mesh& m, const PitchGraph& g, double T, Tents& out, void*
     p.nv = nv;
     p.vpb = (int)(vpt * kPitchThreads);
     p.T = T;
-    // a list holds every round's tents of a block: at most every vertex once a round; bounded memory
-    p.max_rounds = (int)std::max<int64_t>(8, std::min<int64_t>(kPitchChunk, ((int64_t)1 << 25) / nv));
-    p.cap = (int64_t)p.vpb * p.max_rounds;
+    p.max_rounds = kPitchChunk;
+    p.cap = (int64_t)p.vpb * kPitchList;
     PitchBuffers B;
     int64_t *d_ptr, *d_out_off, *d_list_off, *d_round_end;
     int32_t *d_dst, *o_v;
@@ -288,7 +294,7 @@ int device_pitch(const Mesh& m, const PitchGraph& g, double T, Tents& out, void*
     long long rounds = 0;
     while (true) {
         h.arrived = h.released = 0;
-        h.rounds = 0;
+        h.rounds = h.full = h.stop = 0;
         PITCH_TRY(cudaMemcpyAsync(p.ctl, &h, sizeof(h), cudaMemcpyHostToDevice, st));
         void* args[] = {&p};
         PITCH_TRY(cudaLaunchCooperativeKernel((const void*)pitch_rounds_kernel, dim3(nblocks), dim3(kPitchThreads), args, 0, st));
