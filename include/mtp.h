@@ -168,9 +168,14 @@ int mtp_state_to_lattice(mtp_mesh_t mesh, const void* state_dev, double* vals_de
 int mtp_evolve(mtp_tents_t tents, void* state_dev, double T, void* stream);
 
 /* Evolve launch configuration of this tents handle: 0 (default) the persistent DAG walk with as
- * many CTAs per SM as fit and as the average layer fills, 1 the DAG walk with one CTA per SM, 2 one launch per layer (CUDA
- * graph).  MTP_FLAG_LAYER_LAUNCHES on the mesh forces 2. */
+ * many CTAs per SM as fit and as the layers fill (mtp_tents_walk), 1 the DAG walk with one CTA per SM, 2 one
+ * launch per layer (CUDA graph).  MTP_FLAG_LAYER_LAUNCHES on the mesh forces 2. */
 int mtp_tents_set_launch(mtp_tents_t tents, int launch);
+
+/* What an evolve of all layers in launch configuration 0 takes on a GPU of `sms` SMs where `fit` CTAs of the
+ * tent kernel fit on one: CTAs per SM, and the item shape of the kernel (the variant of the handle, or the
+ * one that MTP_FP32_SPLIT chooses in 3D up to p = 3).  Host only. */
+int mtp_tents_walk(mtp_tents_t tents, int sms, int fit, int* ctas, int* shape);
 
 /* Kernel shape variant of this tents handle (MTP_FP32 SAT meshes).  In 2D, and in 3D up to p = 4,
  * variants 0, 1 and 2 all select the apex tent kernel, which is the fastest for every layer width,

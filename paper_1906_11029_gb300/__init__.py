@@ -29,7 +29,7 @@ _CODES = {0: "MTP_OK", -1: "MTP_EINVAL", -2: "MTP_EMESH", -3: "MTP_ECAUSAL", -4:
 ABI_SYMBOLS = ["mtp_mesh_create", "mtp_mesh_destroy", "mtp_mesh_info", "mtp_pitch_tents", "mtp_pitch_tents_device",
                "mtp_tents_destroy", "mtp_tents_info", "mtp_tents_get", "mtp_state_from_lattice",
                "mtp_state_to_lattice", "mtp_evolve", "mtp_evolve_layers", "mtp_evolve_host",
-               "mtp_tents_set_launch", "mtp_tents_set_variant", "mtp_tents_autotune", "mtp_batch_create", "mtp_batch_destroy", "mtp_batch_info", "mtp_batch_evolve",
+               "mtp_tents_set_launch", "mtp_tents_walk", "mtp_tents_set_variant", "mtp_tents_autotune", "mtp_batch_create", "mtp_batch_destroy", "mtp_batch_info", "mtp_batch_evolve",
                "mtp_adjoint", "mtp_energy", "mtp_energy_noalloc", "mtp_probe_rates", "mtp_last_error"]
 
 
@@ -65,6 +65,7 @@ def _load():
         "mtp_evolve_layers": (C.c_int, [P, P, I64, I64, P]),
         "mtp_evolve_host": (C.c_int, [P, P, P, D, P]),
         "mtp_tents_set_launch": (C.c_int, [P, C.c_int]),
+        "mtp_tents_walk": (C.c_int, [P, C.c_int, C.c_int, P, P]),
         "mtp_tents_set_variant": (C.c_int, [P, C.c_int]),
         "mtp_tents_autotune": (C.c_int, [P, P, I64, I64, P, P, P]),
         "mtp_batch_create": (C.c_int, [I64, P, C.POINTER(P)]),
@@ -198,6 +199,13 @@ def mtp_evolve_host(tents, state_in, state_out, T, stream=None):
 
 def mtp_tents_set_launch(h, launch):
     _check(_lib.mtp_tents_set_launch(h, launch))
+
+
+def mtp_tents_walk(h, sms, fit):
+    """(CTAs per SM, item shape) of an evolve on a GPU of ``sms`` SMs where ``fit`` CTAs fit on one."""
+    ctas, shape = C.c_int(), C.c_int()
+    _check(_lib.mtp_tents_walk(h, sms, fit, C.byref(ctas), C.byref(shape)))
+    return ctas.value, shape.value
 
 
 def mtp_tents_set_variant(h, variant):

@@ -518,19 +518,12 @@ static int device_tents_upload(Tents& t) {
     return MTP_OK;
 }
 
-// Shape variant of the tents' kernel: the caller's, and in the 3D split mode, which has no variants to
-// choose from, the one that is faster for the layers (the same bits either way).  Shape 2 wins while a
-// layer is at most a CTA per SM and a row of it is short: 60 layers of 143 tents (p = 1, 2, 3) 1.68, 3.75,
-// 10.0 ms with shape 1 against 1.48, 3.38, 9.7 ms; of 240 tents 1.70, 4.34, 13.1 against 2.23, 5.11, 14.4.
-// At p = 4 shape 2 loses everywhere (27 ms against 38 ms).
+// item shape of the tents' kernel on the current device
 static int item_shape(const Tents& t) {
-    const Mesh& m = *t.mesh;
-    if (m.precision != MTP_FP32_SPLIT || m.dim != 3 || m.p > 3) return t.variant;
     int dev = 0, nsm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
+    if (t.mesh->precision != MTP_FP32_SPLIT || cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return t.variant;
-    const int64_t layers = (int64_t)t.layer_ptr.size() - 1;
-    return (int64_t)t.vertex.size() <= nsm * layers ? 2 : t.variant;
+    return walk_shape(t, nsm);
 }
 
 // general tent kernels
@@ -710,12 +703,7 @@ int device_evolve(Tents& t, void* state, int64_t lb, int64_t le, bool use_graph,
         CUDA_TRY(ke.persistent_prepare(m.max_patch, &bpsm));
         CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
         const int64_t t0 = t.layer_ptr[lb], nt = t.layer_ptr[le] - t0;
-        // as many CTAs per SM as fit, but no more than the layers fill: CTAs beyond the tents of a
-        // layer only wait, and leave the running ones unevenly spread over the SMs (cavity 16^3,
-        // p = 3, 133 tents per layer: 73 us per layer with 3 CTAs per SM, 61 us with one)
-        const double width = (double)nt / (double)(le - lb);
-        const int fill = (int)std::min(64.0, std::ceil(width / nsm));
-        const int cps = launch == 1 ? 1 : std::max(1, std::min(bpsm, fill));
+        const int cps = launch == 1 ? 1 : walk_ctas(t, lb, le, nsm, bpsm);
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t)cps * nsm));
         if (lb == 0) {
             CUDA_TRY(cudaMemsetAsync(d.cnt, 0, sizeof(int) * m.nv, st));

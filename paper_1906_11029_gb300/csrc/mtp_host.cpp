@@ -431,6 +431,53 @@ void pitch_finish(const Mesh& m, double T, double cf, Tents& out) {
     out.cf = cf;
 }
 
+// Rounds that the average layer takes when `slots` of its tents run at a time, one at least.
+static double layer_rounds(const Tents& t, int64_t lb, int64_t le, int64_t slots) {
+    double s = 0;
+    for (int64_t l = lb; l < le; ++l) s += std::fmax(1.0, (double)(t.layer_ptr[l + 1] - t.layer_ptr[l]) / (double)slots);
+    return s / (double)std::max<int64_t>(1, le - lb);
+}
+
+// CTAs per SM of the DAG walk, at most `fit`.  CTAs beyond the tents of a layer only wait, and leave the running
+// ones unevenly spread over the SMs, so one more per SM is added only while it saves at least a certain part of
+// the rounds that it would save on wide layers: a fifth, and from p = 3 on, where two tents of an SM take longer than
+// one, 27 %.  Rounds, not the average width, since a few small elements make many
+// narrow layers, while most tents stay in wide ones.  Measured on 152 SMs with 1 | 2 CTAs per SM, for
+// r = rounds with one / rounds with two (the lines are at 1.11 and 1.16):
+//   cube 16^3, r 1.02 (133 tents a layer), p = 3 in FP32      61 | 73 us a layer (3 CTAs)
+//   16^3 with one vertex near its neighbour, r 1.09 (50), p = 2, 3      23.7, 58.0 | 24.7, 65.4 ms
+//   cube 16^3, a short slab, r 1.14 (146), p = 1 .. 4      1.67, 3.37, 8.2, 21.9 | 1.30, 3.14, 8.4, 23.4 ms
+//   cube 17^3, r 1.20 (168), p = 1 .. 4      3.7, 7.4, 17.7, 46.5 | 2.6, 6.3, 17.0, 47.6 ms
+//   graded 13^3, r 1.23 (156), p = 2, 3, 4      3.5, 8.3, 22.6 | 2.9, 7.8, 21.9 ms
+//   20^3 with one vertex near its neighbour, r 1.31 (144), p = 2, 3      25.8, 62.8 | 22.7, 61.6 ms
+//   32^3 likewise, r 1.57 (344), p = 2, 4      115, 812 | 84, 697 ms
+int walk_ctas(const Tents& t, int64_t lb, int64_t le, int nsm, int fit) {
+    const double part = t.mesh->p <= 2 ? 0.2 : 0.27;
+    int c = 1;
+    double now = layer_rounds(t, lb, le, nsm);
+    while (c < fit) {
+        const double more = layer_rounds(t, lb, le, (int64_t)(c + 1) * nsm);
+        if (now - more < part * now / (c + 1)) break;
+        now = more;
+        ++c;
+    }
+    return c;
+}
+
+// Shape variant of the tents' kernel: the caller's, and in the 3D split mode, which has no variants to choose
+// from, the one that is faster for the layers (the same bits either way): shape 2, one CTA per SM, while a second
+// one would save little.  With r as above, shape 1 | 2: 17^3, r 1.20, p = 1, 2, 3      6.9, 17.6, 53.2 | 6.9, 15.9,
+// 45.3 ms; 18^3, r 1.32      7.7, 19.7, 59.9 | 8.4, 19.3, 54.7 ms; 20^3, r 1.52      5.4, 13.8, 42.2 | 6.8, 15.6, 44.4 ms;
+// 20^3 with one vertex near its neighbour, r 1.31      7.4, 19.1, 56.4 | 7.8, 18.5, 53.5 ms; 32^3 likewise, r 1.57,
+// p = 2, 3      71, 214 | 83, 238 ms.  At p = 4 shape 2 loses everywhere.
+int walk_shape(const Tents& t, int nsm) {
+    const Mesh& m = *t.mesh;
+    if (m.precision != MTP_FP32_SPLIT || m.dim != 3 || m.p > 3) return t.variant;
+    const int64_t nl = (int64_t)t.layer_ptr.size() - 1;
+    const double r = layer_rounds(t, 0, nl, nsm) / layer_rounds(t, 0, nl, 2 * (int64_t)nsm);
+    return r <= (m.p == 1 ? 1.15 : 1.35) ? 2 : t.variant;
+}
+
 }  // namespace mtp
 
 // =================================================================================
@@ -614,6 +661,15 @@ int mtp_tents_set_launch(mtp_tents_t tents, int launch) {
     if (!tents) return set_error(MTP_EINVAL, "tents is NULL");
     if (launch < 0 || launch > 2) return set_error(MTP_EINVAL, "launch must be 0, 1 or 2");
     tents->t.launch = launch;
+    return MTP_OK;
+}
+
+int mtp_tents_walk(mtp_tents_t tents, int sms, int fit, int* ctas, int* shape) {
+    if (!tents || !ctas || !shape) return set_error(MTP_EINVAL, "NULL argument");
+    if (sms < 1 || fit < 1) return set_error(MTP_EINVAL, "sms and fit must be positive");
+    const Tents& t = tents->t;
+    *ctas = walk_ctas(t, 0, (int64_t)t.layer_ptr.size() - 1, sms, fit);
+    *shape = walk_shape(t, sms);
     return MTP_OK;
 }
 

@@ -115,6 +115,10 @@ struct Tents {
     struct DeviceTents* dev = nullptr;
 };
 
+// launch choices of the walk over layers [lb, le) on `nsm` SMs (see the definitions)
+int walk_ctas(const Tents& t, int64_t lb, int64_t le, int nsm, int fit);
+int walk_shape(const Tents& t, int nsm);
+
 struct Batch {
     std::vector<Tents*> inst;
     std::vector<int32_t> ticket_inst;
