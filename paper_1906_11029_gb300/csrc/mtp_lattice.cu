@@ -88,8 +88,7 @@ __global__ void __launch_bounds__(LatShape<DIM, P>::NT) from_lattice_kernel(cons
 
 // Few elements: a thread per value with the dense products, in the order of the points or functions, which
 // spreads them over all SMs.  The kernels above take as long for one CTA as for one on every SM: in FP32
-// at degree 4, 45 / 55 us to / from the lattice with 96 CTAs (3072 elements); these take 17 / 24 us for 384
-// elements, of which 14 / 23 us are the call.
+// at degree 4, 40 / 46 us to / from the lattice (device time); these take 14 / 10 us for 384 elements.
 template <typename Real>
 __global__ void __launch_bounds__(128) to_lattice_small_kernel(const Real* state, double* vals, const double* geo, const double* V,
                                                                int64_t ne, int nf, int nb, int64_t n) {
@@ -197,16 +196,26 @@ __global__ void energy_final_kernel(const double* partial, int nblocks, double* 
     if (threadIdx.x == 0) out[rhs] = 0.5 * red[0];
 }
 
-// CTAs for n elements: no more than can be resident, so that a CTA's loop amortises its launch
-int lattice_grid(int64_t n) {
-    const int64_t g = (n + kLatElems - 1) / kLatElems;
-    return (int)(g < 152 * 32 ? g : 152 * 32);
+cudaError_t sm_count(int* n) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e != cudaSuccess ? e : cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev);
 }
 
-// Elements up to which the small kernels run: while the others leave half of the SMs without a CTA.  There the
-// two take the same time (2058 elements of degree 4, FP32, to the lattice: 64 us with the small kernel, 3072
-// elements 91 us with it and 45 us with the other).
-constexpr int64_t kSmallElems = 16 * 152;
+// CTAs for n elements: no more than can be resident, so that a CTA's loop amortises its launch
+int lattice_grid(int64_t n, int nsm) {
+    const int64_t g = (n + kLatElems - 1) / kLatElems;
+    return (int)(g < nsm * 32 ? g : nsm * 32);
+}
+
+// Elements per SM up to which the small kernels run.  They are as fast as the others, in 3D at degrees 3, 4 and 5 on
+// 152 SMs, for about 2700 elements (18 per SM), from the lattice in both precisions and to the lattice in FP64: 14 | 14,
+// 36 | 37, 86 | 88 us for 2688 elements with the small | the other kernel, to the lattice in FP64; 19 | 19, 45 | 46,
+// 106 | 105 us from it in FP32.  To the lattice in FP32 every product of theirs converts its coefficient, and the
+// line is at 1300 elements: 13 | 15, 34 | 40, 81 | 93 us for 1152, 19 | 15, 54 | 41, 134 | 93 us for 1920.
+template <typename Real>
+constexpr int kSmallTo = sizeof(Real) == 4 ? 8 : 16;
+constexpr int kSmallFrom = 16;
 
 template <typename K>
 cudaError_t lattice_smem(K kernel, size_t bytes) {
@@ -219,20 +228,26 @@ struct Lattice {
     static cudaError_t to(const Mesh& m, const void* state, double* vals, cudaStream_t st) {
         constexpr size_t bytes = (size_t)kLatElems * Sh::SP * sizeof(double);
         const int64_t n = (int64_t)m.n_rhs * m.ne;
-        if (n <= kSmallElems) {
+        int nsm = 0;
+        cudaError_t e = sm_count(&nsm);
+        if (e != cudaSuccess) return e;
+        if (n <= (int64_t)kSmallTo<Real> * nsm) {
             to_lattice_small_kernel<Real><<<(unsigned)((n * Sh::NC + 127) / 128), 128, 0, st>>>(
                 (const Real*)state, vals, device_geo(m), device_lattice_tables(m)[0], m.ne, Sh::NF, Sh::NB, n * Sh::NC);
             return cudaGetLastError();
         }
-        const cudaError_t e = lattice_smem(to_lattice_kernel<Real, DIM, P>, bytes);
+        e = lattice_smem(to_lattice_kernel<Real, DIM, P>, bytes);
         if (e != cudaSuccess) return e;
-        to_lattice_kernel<Real, DIM, P><<<lattice_grid(n), Sh::NT, bytes, st>>>((const Real*)state, vals, device_geo(m), m.ne, n);
+        to_lattice_kernel<Real, DIM, P><<<lattice_grid(n, nsm), Sh::NT, bytes, st>>>((const Real*)state, vals, device_geo(m), m.ne, n);
         return cudaGetLastError();
     }
     static cudaError_t from(const Mesh& m, const double* vals, void* state, cudaStream_t st) {
         constexpr size_t bytes = (size_t)kLatElems * Sh::SP * sizeof(double);
         const int64_t n = (int64_t)m.n_rhs * m.ne;
-        if (n <= kSmallElems) {
+        int nsm = 0;
+        cudaError_t e = sm_count(&nsm);
+        if (e != cudaSuccess) return e;
+        if (n <= (int64_t)kSmallFrom * nsm) {
             from_lattice_small_kernel<Real><<<(unsigned)((n * Sh::NC + 127) / 128), 128, 0, st>>>(
                 vals, (Real*)state, device_geo(m), device_lattice_tables(m)[1], m.ne, Sh::NF, Sh::NB, n * Sh::NC);
             return cudaGetLastError();
@@ -242,9 +257,9 @@ struct Lattice {
             from_lattice_dense_kernel<Real><<<(unsigned)(g < 65535 ? g : 65535), 256, 0, st>>>(
                 vals, (Real*)state, device_geo(m), device_lattice_tables(m)[1], m.ne, Sh::NF, Sh::NB, rows);
         } else {
-            const cudaError_t e = lattice_smem(from_lattice_kernel<Real, DIM, P>, bytes);
+            e = lattice_smem(from_lattice_kernel<Real, DIM, P>, bytes);
             if (e != cudaSuccess) return e;
-            from_lattice_kernel<Real, DIM, P><<<lattice_grid(n), Sh::NT, bytes, st>>>(vals, (Real*)state, device_geo(m), m.ne, n);
+            from_lattice_kernel<Real, DIM, P><<<lattice_grid(n, nsm), Sh::NT, bytes, st>>>(vals, (Real*)state, device_geo(m), m.ne, n);
         }
         return cudaGetLastError();
     }
