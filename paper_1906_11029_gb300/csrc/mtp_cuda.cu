@@ -529,8 +529,8 @@ static int item_shape(const Tents& t) {
 // general tent kernels
 static const KernelEntry& general_entry(const Mesh& m, int variant) {
     static KernelEntry f64[2][5], f32[2][5], tc[2][5], split[2][5], narrow[3], rk4[2][5], f32v1[2][5], f32v2[2][5], tc5[2][5];
-    static bool init = false;
-    if (!init) {
+    static std::once_flag once;   // calls come from several threads
+    std::call_once(once, [] {
         kernel_table_f32_tc5(tc5);
         kernel_table_f64(f64);
         kernel_table_f32(f32);
@@ -540,8 +540,7 @@ static const KernelEntry& general_entry(const Mesh& m, int variant) {
         kernel_table_rk4(rk4);
         kernel_table_f32_v1(f32v1);
         kernel_table_f32_v2(f32v2);
-        init = true;
-    }
+    });
     if ((variant == 3 || variant == 4) && m.precision == MTP_FP32 && m.dim == 3 && !(m.flags & MTP_FLAG_SUBSTITUTED_RK4))
         return tc5[variant - 3][m.p - 1];   // null entries outside p = 2..4 (refused when the variant is set)
     if (variant == 2 && m.precision == MTP_FP32 && !(m.flags & MTP_FLAG_SUBSTITUTED_RK4))
@@ -570,8 +569,8 @@ static bool apex_runs(const Mesh& m, int variant) {
 static const KernelEntry& kernel_entry(const Mesh& m, int variant = 0) {
     if (!apex_runs(m, variant)) return general_entry(m, variant);
     static KernelEntry apex[2][2][5];
-    static bool init = false;
-    if (!init) {
+    static std::once_flag once;   // calls come from several threads
+    std::call_once(once, [] {
         for (int p = 1; p <= 5; ++p) {
             apex[0][0][p - 1] = apex2_entry_f64(p);
             apex[1][0][p - 1] = apex2_entry_f32(p);
@@ -579,8 +578,7 @@ static const KernelEntry& kernel_entry(const Mesh& m, int variant = 0) {
             apex[0][1][p - 1] = apex_entry_f64(p);
             apex[1][1][p - 1] = apex_entry_f32(p);
         }
-        init = true;
-    }
+    });
     return apex[m.precision == MTP_FP64 ? 0 : 1][m.dim - 2][m.p - 1];
 }
 
@@ -826,8 +824,8 @@ int device_adjoint(Tents& t, const void* state0, const void* lamT, void* lam0, d
     DeviceTents& d = *t.dev;
     cudaStream_t st = (cudaStream_t)stream;
     static AdjEntry general[2][2][5], apex[2][5];
-    static bool init = false;
-    if (!init) { adjoint_table(general); apex_adjoint_table(apex); init = true; }
+    static std::once_flag once;
+    std::call_once(once, [] { adjoint_table(general); apex_adjoint_table(apex); });
     if (m.precision == MTP_FP32_SPLIT || (m.flags & MTP_FLAG_SUBSTITUTED_RK4))
         return set_error(MTP_EUNSUPPORTED, "the adjoint runs SAT meshes in FP64, FP32 or a tensor-core mode");
     const int fp = m.precision == MTP_FP64 ? 0 : 1;   // the tensor-core modes' adjoint runs in FP32
@@ -991,8 +989,8 @@ int device_batch_evolve(Batch& b, void* const* states, void* stream) {
     for (Tents* t : b.inst) MTP_TRY(device_tents_upload(*t));
     const Mesh& m0 = *b.inst[0]->mesh;
     static BatchEntry general[2][2];
-    static bool init = false;
-    if (!init) { batch_table(general); init = true; }
+    static std::once_flag once;
+    std::call_once(once, [] { batch_table(general); });
     for (Tents* t : b.inst)
         if (t->mesh->flags & MTP_FLAG_SUBSTITUTED_RK4)
             return set_error(MTP_EUNSUPPORTED, "batches run SAT meshes; MTP_FLAG_SUBSTITUTED_RK4 is per mesh");
