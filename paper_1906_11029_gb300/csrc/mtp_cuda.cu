@@ -372,16 +372,8 @@ static int apex_upload(const Mesh& m) {
     return rc;
 }
 
-int device_mesh_upload(Mesh& m) {
-    int dev;
-    CUDA_TRY(cudaGetDevice(&dev));
-    if (m.dev) {
-        if (m.dev->device == dev) return MTP_OK;
-        return set_error(MTP_EINVAL, "mesh was uploaded to another device");
-    }
-    m.dev = new DeviceMesh();
+static int mesh_buffers(Mesh& m) {
     DeviceMesh& d = *m.dev;
-    d.device = dev;
     MTP_TRY(upload(&d.geo, m.geo.data(), m.geo.size()));
     MTP_TRY(upload(&d.lattice[0], m.ref.V.data(), m.ref.V.size()));
     MTP_TRY(upload(&d.lattice[1], m.ref.Vinv.data(), m.ref.Vinv.size()));
@@ -457,7 +449,28 @@ int device_mesh_upload(Mesh& m) {
         MTP_TRY(upload(&d.Trf_lo, tl.data(), tl.size()));
     }
     CUDA_TRY(cudaMalloc((void**)&d.partial, sizeof(double) * energy_scratch_doubles(m)));
+    CUDA_TRY(cudaStreamSynchronize(0));   // the copies: the first kernels may run on any stream
     return MTP_OK;
+}
+
+// The mesh's device copies, made by the first call, whichever thread it comes from.  Where one of them has no room, all
+// are given back and the next call tries again: nothing may run with some of them missing.
+int device_mesh_upload(Mesh& m) {
+    int dev;
+    CUDA_TRY(cudaGetDevice(&dev));
+    static std::mutex lock;
+    std::lock_guard<std::mutex> guard(lock);
+    if (m.dev) {
+        if (m.dev->device == dev) return MTP_OK;
+        return set_error(MTP_EINVAL, "mesh was uploaded to another device");
+    }
+    m.dev = new DeviceMesh();
+    m.dev->device = dev;
+    const int rc = mesh_buffers(m);
+    if (rc == MTP_OK) return rc;
+    device_mesh_free(m);
+    cudaGetLastError();
+    return rc;
 }
 
 void device_mesh_free(Mesh& m) {
@@ -486,10 +499,7 @@ void device_tents_free(Tents& t) {
     t.dev = nullptr;
 }
 
-static int device_tents_upload(Tents& t) {
-    MTP_TRY(device_mesh_upload(*t.mesh));
-    if (t.dev) return MTP_OK;
-    t.dev = new DeviceTents();
+static int tents_buffers(Tents& t) {
     DeviceTents& d = *t.dev;
     MTP_TRY(upload(&d.v, t.vertex.data(), t.vertex.size()));
     MTP_TRY(upload(&d.tb, t.t_bot.data(), t.t_bot.size()));
@@ -515,7 +525,20 @@ static int device_tents_upload(Tents& t) {
     MTP_TRY(upload(&d.adj, m.adj.data(), m.adj.size()));
     CUDA_TRY(cudaMalloc((void**)&d.cnt, sizeof(int) * m.nv));
     CUDA_TRY(cudaMalloc((void**)&d.next, sizeof(unsigned long long)));
+    CUDA_TRY(cudaStreamSynchronize(0));
     return MTP_OK;
+}
+
+// all or nothing, as device_mesh_upload
+static int device_tents_upload(Tents& t) {
+    MTP_TRY(device_mesh_upload(*t.mesh));
+    if (t.dev) return MTP_OK;
+    t.dev = new DeviceTents();
+    const int rc = tents_buffers(t);
+    if (rc == MTP_OK) return rc;
+    device_tents_free(t);
+    cudaGetLastError();
+    return rc;
 }
 
 // item shape of the tents' kernel on the current device
@@ -983,6 +1006,23 @@ void device_batch_free(Batch& b) {
     b.dev = nullptr;
 }
 
+static int batch_buffers(Batch& b) {
+    DeviceBatch& d = *b.dev;
+    const int64_t ni = (int64_t)b.inst.size();
+    MTP_TRY(upload(&d.ticket_inst, b.ticket_inst.data(), b.ticket_inst.size()));
+    MTP_TRY(upload(&d.ticket_tent, b.ticket_tent.data(), b.ticket_tent.size()));
+    std::vector<int32_t> ps(ni);
+    for (int64_t i = 0; i < ni; ++i) ps[i] = b.inst[i]->mesh->p;
+    MTP_TRY(upload(&d.inst_p, ps.data(), ps.size()));
+    CUDA_TRY(cudaMalloc((void**)&d.kargs, sizeof(KArgs) * ni));
+    CUDA_TRY(cudaMalloc((void**)&d.pargs, sizeof(PArgs) * ni));
+    CUDA_TRY(cudaMalloc((void**)&d.next, sizeof(unsigned long long)));
+    CUDA_TRY(cudaMalloc((void**)&d.err, sizeof(int)));
+    CUDA_TRY(cudaMallocHost((void**)&d.err_host, sizeof(int)));
+    CUDA_TRY(cudaStreamSynchronize(0));
+    return MTP_OK;
+}
+
 int device_batch_evolve(Batch& b, void* const* states, void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
     const int64_t ni = (int64_t)b.inst.size();
@@ -1019,17 +1059,12 @@ int device_batch_evolve(Batch& b, void* const* states, void* stream) {
     const size_t smem = smem_of(be);
     if (!b.dev) {
         b.dev = new DeviceBatch();
-        DeviceBatch& d = *b.dev;
-        MTP_TRY(upload(&d.ticket_inst, b.ticket_inst.data(), b.ticket_inst.size()));
-        MTP_TRY(upload(&d.ticket_tent, b.ticket_tent.data(), b.ticket_tent.size()));
-        std::vector<int32_t> ps(ni);
-        for (int64_t i = 0; i < ni; ++i) ps[i] = b.inst[i]->mesh->p;
-        MTP_TRY(upload(&d.inst_p, ps.data(), ps.size()));
-        CUDA_TRY(cudaMalloc((void**)&d.kargs, sizeof(KArgs) * ni));
-        CUDA_TRY(cudaMalloc((void**)&d.pargs, sizeof(PArgs) * ni));
-        CUDA_TRY(cudaMalloc((void**)&d.next, sizeof(unsigned long long)));
-        CUDA_TRY(cudaMalloc((void**)&d.err, sizeof(int)));
-        CUDA_TRY(cudaMallocHost((void**)&d.err_host, sizeof(int)));
+        const int rc = batch_buffers(b);
+        if (rc != MTP_OK) {
+            device_batch_free(b);
+            cudaGetLastError();
+            return rc;
+        }
     }
     DeviceBatch& d = *b.dev;
     std::vector<KArgs> ka(ni);
