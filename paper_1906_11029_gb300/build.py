@@ -25,7 +25,7 @@ NVCC = os.path.join(CUDA_HOME, "bin", "nvcc")
 GENCODE = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CXX_SOURCES = ["mtp_host.cpp", "mtp_tables.cpp"]
 CU_SOURCES = ["mtp_cuda.cu", "mtp_lattice.cu", "mtp_k64.cu", "mtp_k32.cu", "mtp_ka32.cu", "mtp_ka64.cu", "mtp_kab32.cu", "mtp_kab64.cu", "mtp_ka2d32.cu", "mtp_ka2d64.cu", "mtp_ks.cu", "mtp_ks2.cu", "mtp_krk.cu", "mtp_kv.cu", "mtp_kv2.cu", "mtp_ktc5.cu", "mtp_ktc.cu", "mtp_kb.cu", "mtp_adj.cu", "mtp_probe.cu", "mtp_noalloc.cu", "mtp_pitch.cu"]
-HEADERS = ["mtp_internal.h", "mtp_device.h", "mtp_kernels.cuh", "mtp_apex.cuh", "mtp_apex2.cuh", "mtp_apex_adjoint.cuh", "mtp_apex_launch.cuh", "mtp_adjoint.cuh", "mtp_launch.cuh", "../../include/mtp.h"]
+HEADERS = ["mtp_internal.h", "mtp_device.h", "mtp_kernels.cuh", "mtp_apex.cuh", "mtp_apex2.cuh", "mtp_apex_adjoint.cuh", "mtp_apex_launch.cuh", "mtp_apex2_launch.cuh", "mtp_adjoint.cuh", "mtp_launch.cuh", "../../include/mtp.h"]
 
 
 def _newer(src_list, target):
