@@ -45,6 +45,16 @@ TRAFFIC_BYTES_PER_TENT = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum on the launch that applies layers
     # 1000..1099 (81 105 tents) of the graded 32^3 p = 4 workload: 1.145 GB + 0.757 GB
     ("fp32", "tent_persistent_kernel"): {"bytes_per_tent": 23455.2, "sources": "215962c12a1e8c1c"},
+    # the same window, layers 1000..1099: 1.642 GB + 0.789 GB
+    ("fp32", "apex_persistent_kernel"): {"bytes_per_tent": 29979.5, "sources": "0fcd0cd9736f146b"},
+}
+
+# Floating-point operations (a fused multiply-add is two) per DOF-update that the apex kernel executes: its operators are
+# sparse, so the dense algorithmic count is about three times that.  By degree, from the FMA, add and multiply counters of
+# the same captures (all 32 lanes of a warp count, also where the patch has fewer elements), stamped like the traffic.
+EXECUTED_FLOP_PER_DOF = {
+    # 738.9e9 FMA, 169.9e9 add, 243.8e9 multiply for 1.4775e10 DOF-updates
+    ("fp32", "apex_persistent_kernel", 4): {"flop": 128.0, "sources": "0fcd0cd9736f146b"},
 }
 
 
@@ -68,6 +78,13 @@ def traffic_per_tent(precision, kernel):
     if rec is None or rec["sources"] != kernel_source_hash():
         return None
     return rec["bytes_per_tent"]
+
+
+def executed_flop_per_dof(precision, kernel, p):
+    rec = EXECUTED_FLOP_PER_DOF.get((precision, kernel, p))
+    if rec is None or rec["sources"] != kernel_source_hash():
+        return None
+    return rec["flop"]
 
 
 def load_peaks():
@@ -584,23 +601,25 @@ def run_mtp(args):
     # roofline of the tent kernel (the evolve is the tent-kernel graph); denominators: the FMA
     # rates measured on this device by mtp_probe_rates (before the timed region), next to the
     # unit-count figure from the device's SM count and maximum clock
-    fl = flops_per_dof_update(w.dim, w.p)
+    dense = flops_per_dof_update(w.dim, w.p)
     launch_ms = kern_ms / (args.steps * launches_per_step)
-    flops_per_launch = dofs * fl / launches_per_step
     n_sms = torch.cuda.get_device_properties(local).multi_processor_count
     unit_peak = n_sms * FP32_SM_LANES * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
     if prec == mtp.MTP_FP32:
         peak, src = probe["fp32_fma"], "mtp_probe_rates FP32 FMA loop on this device, this run"
     else:
         peak, src = probe["fp64_fma"], "mtp_probe_rates FP64 FMA loop on this device, this run"
-    achieved = flops_per_launch / (launch_ms / 1e3) / 1e12
     kname = tent_kernel_name(args.precision, args.variant, w.dim, w.p, persistent)
+    executed = executed_flop_per_dof(args.precision, kname, w.p)
+    dense_tflops = dofs * dense / launches_per_step / (launch_ms / 1e3) / 1e12
+    achieved = dense_tflops if executed is None else dense_tflops * executed / dense
     # the stored traffic is the default kernel's (variant 0, occupancy-limit DAG walk)
     default_kernel = args.variant == 0 and args.launch == 0
     tpl = traffic_per_tent(args.precision, kname) if args.workload == "graded" and default_kernel else None
     traffic = None if tpl is None else tpl * tents.info["n_tents"] / launches_per_step
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic,
+                "flop_count": "dense algorithmic" if executed is None else "executed", "dense_tflops": dense_tflops,
                 "kernel": f"{kname}<{args.precision},3,{w.p}>", "kernel_variant": args.variant, "launch": args.launch, "peak_source": src,
                 "probe_tflops": probe, "fp32_unit_count_peak": unit_peak, "sms": n_sms,
                 "frac_of_unit_count_peak": achieved / unit_peak if prec == mtp.MTP_FP32 else None,

@@ -9,7 +9,8 @@ Two levels:
   kernels or the tensor-core 3xTF32 split; for "tf32" accuracy additionally plain TF32 tensor
   cores;
 * kernel shape of the SIMT FP32 kernels (here, `mtp_tents_set_variant`): variants 0, 1 and 2 are
-  the apex tent kernels in 2D and in 3D up to p = 4; beyond, stage items over pairs
+  the apex tent kernels in 2D and in 3D up to p = 4 (the same kernel: whichever is timed fastest is right); beyond,
+  and on stretched meshes, stage items over pairs
   of patch elements (variant 0), single elements (variant 1) or single (element, row) pairs on
   512 threads (variant 2): more and shorter items, faster tents when the layers hold fewer
   tents than the GPU has CTA slots; variants 3 and 4 (3D, p = 2..4) take the item shapes of 1
